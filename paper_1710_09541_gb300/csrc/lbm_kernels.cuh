@@ -141,6 +141,51 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
     return r;
 }
 
+// Pairs of values that take the same operations: (x, y) components, and the
+// directions (1, 2), (3, 4), (5, 6), (7, 8).  PK = true issues each pair as one
+// packed instruction (add / mul / fma.rn.f32x2), PK = false as two scalar ones;
+// both round each half to nearest, so the bits are the same.
+struct F2 {
+    float x, y;
+};
+__device__ __forceinline__ F2 both(float v) { return F2{v, v}; }
+__device__ __forceinline__ F2 dirs(const float v[9], int i) { return F2{v[i], v[i + 1]}; }
+__device__ __forceinline__ F2 neg(F2 a) { return F2{-a.x, -a.y}; }
+template <bool PK>
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    if constexpr (!PK) return F2{add(a.x, b.x), add(a.y, b.y)};
+    F2 r;
+    asm("{.reg .b64 a, b, d; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; add.rn.f32x2 d, a, b; mov.b64 {%0, %1}, d;}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+template <bool PK>
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    if constexpr (!PK) return F2{mul(a.x, b.x), mul(a.y, b.y)};
+    F2 r;
+    asm("{.reg .b64 a, b, d; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; mul.rn.f32x2 d, a, b; mov.b64 {%0, %1}, d;}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+template <bool PK>
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    if constexpr (!PK) return F2{fma_rn(a.x, b.x, c.x), fma_rn(a.y, b.y, c.y)};
+    F2 r;
+    asm("{.reg .b64 a, b, c, d; mov.b64 a, {%2, %3}; mov.b64 b, {%4, %5}; mov.b64 c, {%6, %7}; "
+        "fma.rn.f32x2 d, a, b, c; mov.b64 {%0, %1}, d;}"
+        : "=f"(r.x), "=f"(r.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return r;
+}
+// a - b: as a fused multiply-add by -1 when packed (exact product, one rounding)
+template <bool PK>
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) {
+    if constexpr (!PK) return F2{sub(a.x, b.x), sub(a.y, b.y)};
+    return fma2<true>(b, both(-1.f), a);
+}
+
 // Programmatic dependent launch.  A step kernel launched with programmatic
 // stream serialisation may be scheduled while the previous step is still
 // finishing: it waits here, before its first access to the state that step
@@ -191,8 +236,10 @@ __device__ __forceinline__ void cdot9(float vx, float vy, float c[9]) {
 // sum of the eight moving populations, in the association order used both
 // for phi below and for the rest population written as the remainder
 // phi - sum8 after the collision
+template <bool PK = false>
 __device__ __forceinline__ float sum8(const float v[9]) {
-    return add(add(add(v[1], v[3]), add(v[2], v[4])), add(add(v[5], v[7]), add(v[6], v[8])));
+    const F2 a = add2<PK>(dirs(v, 1), dirs(v, 3)), d = add2<PK>(dirs(v, 5), dirs(v, 7));
+    return add(add(a.x, a.y), add(d.x, d.y));
 }
 
 // The one-node ring around a TX x TY tile: slot r -> tile-relative (lx, ly),
@@ -224,7 +271,10 @@ struct Ring {
 // own (uniform bulk), f_0 + sum8 then gives back phi exactly (f_0 = phi - sum8
 // is exact by Sterbenz's lemma when sum8 lies in [phi/2, 2 phi]), so the
 // rounding of the two sums cannot drift sum phi in one direction.
-__device__ __forceinline__ float sum9(const float v[9]) { return add(v[0], sum8(v)); }
+template <bool PK = false>
+__device__ __forceinline__ float sum9(const float v[9]) {
+    return add(v[0], sum8<PK>(v));
+}
 
 // coordinate of a tile/halo slot folded into the grid: periodic wrap in x;
 // in y wrap, or clamp at a wall or the open top (ghost row = edge row).
@@ -265,25 +315,30 @@ struct Macro {
 struct GMom {
     float mx, my, snz;
 };
+template <bool PK = false>
 __device__ __forceinline__ GMom gmoments(const float g[9]) {
     GMom o;
-    o.mx = add(sub(g[1], g[3]), add(sub(g[5], g[6]), sub(g[8], g[7])));
-    o.my = add(sub(g[2], g[4]), add(sub(g[5], g[8]), sub(g[6], g[7])));
-    o.snz = add(add(add(g[1], g[3]), add(g[2], g[4])), add(add(g[5], g[7]), add(g[6], g[8])));
+    const F2 d = sub2<PK>(dirs(g, 1), dirs(g, 3));
+    o.mx = add(d.x, add(sub(g[5], g[6]), sub(g[8], g[7])));
+    o.my = add(d.y, add(sub(g[5], g[8]), sub(g[6], g[7])));
+    o.snz = sum8<PK>(g);
     return o;
 }
 
+template <bool PK = false>
 __device__ __forceinline__ Macro macro_from(const Model& m, const GMom& gm, float phi, float gx,
                                             float gy, float lap) {
     Macro o;
     o.rho = fma_rn(phi, m.drho, m.rho_g);                                      // Eq. 13
     const float bulk = mul(mul(mul(m.beta4, phi), sub(phi, 1.f)), sub(phi, 0.5f));
     const float mu = fma_rn(-m.kappa, lap, bulk);                              // Eq. 6
-    o.Fx = fma_rn(mu, gx, m.Gx);                                               // Eqs. 5, 19
-    o.Fy = fma_rn(mu, gy, m.Gy);
+    const F2 F = fma2<PK>(both(mu), F2{gx, gy}, F2{m.Gx, m.Gy});               // Eqs. 5, 19
+    o.Fx = F.x;
+    o.Fy = F.y;
     o.inv_rho = rcp_approx(o.rho);
-    o.ux = mul(fma_rn(0.5f, o.Fx, gm.mx), o.inv_rho);                         // Eq. 22a
-    o.uy = mul(fma_rn(0.5f, o.Fy, gm.my), o.inv_rho);
+    const F2 u = mul2<PK>(fma2<PK>(both(0.5f), F, F2{gm.mx, gm.my}), both(o.inv_rho));  // Eq. 22a
+    o.ux = u.x;
+    o.uy = u.y;
     o.usq = fma_rn(o.ux, o.ux, mul(o.uy, o.uy));
     // Eq. 22b with c_s^2/(1 - w_0) = 3/5 and rho s_0(u) = -(2/3) rho |u|^2
     const float ugrad = fma_rn(o.ux, gx, mul(o.uy, gy));
@@ -302,18 +357,21 @@ __device__ __forceinline__ Macro macroscopic(const Model& m, const float g[9], f
 struct Stencil {
     float gx, gy, lap;
 };
+template <bool PK = false>
 __device__ __forceinline__ Stencil stencil(float pC, float pE, float pW, float pN, float pS,
                                            float pNE, float pNW, float pSW, float pSE) {
     Stencil s;
-    const float dd = sub(pNE, pSW);
-    const float da = sub(pSE, pNW);
-    s.gx = fma_rn(sub(pE, pW), 1.f / 3.f, mul(add(dd, da), 1.f / 12.f));
-    s.gy = fma_rn(sub(pN, pS), 1.f / 3.f, mul(sub(dd, da), 1.f / 12.f));
+    const F2 EN{pE, pN}, WS{pW, pS}, up{pNE, pNW}, dn{pSW, pSE}, C = both(pC);
+    const F2 d = sub2<PK>(up, dn);  // NE - SW, NW - SE
+    const F2 g = fma2<PK>(sub2<PK>(EN, WS), both(1.f / 3.f),
+                          mul2<PK>(F2{sub(d.x, d.y), add(d.x, d.y)}, both(1.f / 12.f)));
+    s.gx = g.x;
+    s.gy = g.y;
     // differences to the centre first: nearly exact in FP32 for neighbouring
     // values (Sterbenz), so the Laplacian carries no O(ulp(phi)) cancellation
-    const float axis = add(add(sub(pE, pC), sub(pW, pC)), add(sub(pN, pC), sub(pS, pC)));
-    const float diag = add(add(sub(pNE, pC), sub(pSW, pC)), add(sub(pNW, pC), sub(pSE, pC)));
-    s.lap = fma_rn(axis, 2.f / 3.f, mul(diag, 1.f / 6.f));
+    const F2 a = add2<PK>(sub2<PK>(EN, C), sub2<PK>(WS, C));
+    const F2 b = add2<PK>(sub2<PK>(up, C), sub2<PK>(dn, C));
+    s.lap = fma_rn(add(a.x, a.y), 2.f / 3.f, mul(add(b.x, b.y), 1.f / 6.f));
     return s;
 }
 
@@ -336,6 +394,7 @@ __device__ __forceinline__ float geq_i(int i, float p3, float rho, float cu, flo
 // Both collisions of one node (Eqs. 2, 3, 8, 9, 11 and 15-17, 20); f and g are
 // overwritten with the post-collision values.  phiu_prev = (phi u) of the
 // previous step.  Returns (phi ux, phi uy) of this step.
+template <bool PK = false>
 __device__ __forceinline__ float2 collide(const Model& m, float f[9], float g[9], float phi,
                                           const Stencil& st, const Macro& M, float2 phiu_prev) {
     const float ux = M.ux, uy = M.uy;
@@ -343,13 +402,11 @@ __device__ __forceinline__ float2 collide(const Model& m, float f[9], float g[9]
     const float nu = viscosity(m, phi, M.inv_rho);
     const float omega_g = rcp_approx(fma_rn(3.f, nu, 0.5f));
 
-    float cu[9];
-    cdot9(ux, uy, cu);
-
     // d_t(phi u) by the backward difference, Eq. 11
-    const float2 phiu = make_float2(mul(phi, ux), mul(phi, uy));
-    const float Dx = sub(phiu.x, phiu_prev.x);
-    const float Dy = sub(phiu.y, phiu_prev.y);
+    const F2 pu = mul2<PK>(both(phi), F2{ux, uy});
+    const F2 D = sub2<PK>(pu, F2{phiu_prev.x, phiu_prev.y});
+    const float2 phiu = make_float2(pu.x, pu.y);
+    const float Dx = D.x, Dy = D.y;
     const float lam = mul(mul(m.four_over_W, phi), sub(1.f, phi));  // Eq. 3
     float nx_ = 0.f, ny_ = 0.f;
     if (!m.local_normal) {  // Eq. 2 with the gradient of Eq. 27
@@ -360,7 +417,8 @@ __device__ __forceinline__ float2 collide(const Model& m, float f[9], float g[9]
             ny_ = mul(st.gy, inv);
         }
     } else {  // Eq. 29: C = sum c_i (f_i - f_i^eq) + d_t(phi u)/2, n = -C/|C|
-        float ne[9];
+        float ne[9], cu[9];
+        cdot9(ux, uy, cu);
 #pragma unroll
         for (int i = 1; i < 9; ++i) ne[i] = sub(f[i], feq_i(i, phi, cu[i]));
         const float Cx = add(mul(0.5f, Dx), add(sub(ne[1], ne[3]), add(sub(ne[5], ne[6]), sub(ne[8], ne[7]))));
@@ -388,14 +446,11 @@ __device__ __forceinline__ float2 collide(const Model& m, float f[9], float g[9]
     // used: it moves every bulk value by an ulp each step, which drifted
     // sum phi 400x more on the layered Poiseuille run (4e-5 over 2e5 steps)
     // and shifted the FP16-stored Laplace jump by 4.6%.
-    const float l3 = mul(lam, 1.f / 3.f);
-    float cv[9], ch[9], ce[9];
-    cdot9(fma_rn(m.tau_f_mh, fma_rn(l3, nx_, Dx), phiu.x),
-          fma_rn(m.tau_f_mh, fma_rn(l3, ny_, Dy), phiu.y), cv);   // c_i . V
+    const F2 V = fma2<PK>(both(m.tau_f_mh), fma2<PK>(both(mul(lam, 1.f / 3.f)), F2{nx_, ny_}, F2{Dx, Dy}),
+                          F2{phiu.x, phiu.y});                        // c_i . V
     const float nu9 = mul(9.f, nu);
-    cdot9(mul(nu9, M.Fx), mul(nu9, M.Fy), ch);                    // c_i . 3 nu 3F
-    const float e9 = mul(nu9, m.drho);
-    cdot9(mul(e9, st.gx), mul(e9, st.gy), ce);                    // c_i . 3 nu 3 (rho_l - rho_g) grad phi
+    const F2 h = mul2<PK>(both(nu9), F2{M.Fx, M.Fy});                 // c_i . 3 nu 3F
+    const F2 e = mul2<PK>(both(mul(nu9, m.drho)), F2{st.gx, st.gy});  // c_i . 3 nu 3 (rho_l - rho_g) grad phi
     const float p3 = mul(3.f, M.p);
     const float m15 = mul(-1.5f, M.usq);
 
@@ -408,16 +463,32 @@ __device__ __forceinline__ float2 collide(const Model& m, float f[9], float g[9]
         const float geq0 = fma_rn(M.rho, mul(w_of(0), m15), mul(p3, w_of(0) - 1.f));
         g[0] = fma_rn(omega_g, sub(geq0, g[0]), g[0]);
     }
+    // directions i, i + 1 (c_i . v = vx, vy for i = 1; vx + vy, vy - vx for
+    // i = 5) and their opposites i + 2, i + 3, whose c_i . v have the other sign
 #pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        // Allen-Cahn, Eqs. 8, 9, 11
-        const float fe = fma_rn(cv[i], 3.f * w_of(i), mul(w_of(i), phi));
-        f[i] = fma_rn(m.inv_tau_f, sub(fe, f[i]), f[i]);
-        // Navier-Stokes, Eqs. 15-17, 20
-        const float s = fma_rn(cu[i], fma_rn(4.5f, cu[i], 3.f), m15);   // s_i / w_i
-        const float t = fma_rn(cu[i], ce[i], ch[i]);
-        const float ge = fma_rn(w_of(i), fma_rn(M.rho, s, t), mul(p3, w_of(i)));
-        g[i] = fma_rn(omega_g, sub(ge, g[i]), g[i]);
+    for (int i = 1; i < 9; i += 4) {
+        const float w = w_of(i);
+        auto cdot = [&](F2 v) { return i == 1 ? v : F2{add(v.x, v.y), sub(v.y, v.x)}; };
+        const F2 cv = cdot(V), ch = cdot(h), ce = cdot(e), c = cdot(F2{ux, uy});
+        const F2 wphi = both(mul(w, phi)), wp3 = both(mul(p3, w));
+#pragma unroll
+        for (int o = 0; o < 2; ++o) {
+            const int j = i + 2 * o;
+            const float sg = o ? -1.f : 1.f;
+            // Allen-Cahn, Eqs. 8, 9, 11
+            const F2 fj = dirs(f, j), gj = dirs(g, j);
+            const F2 fe = fma2<PK>(cv, both(sg * 3.f * w), wphi);
+            const F2 fn = fma2<PK>(both(m.inv_tau_f), sub2<PK>(fe, fj), fj);
+            // Navier-Stokes, Eqs. 15-17, 20
+            const F2 s = fma2<PK>(c, fma2<PK>(both(4.5f), c, both(sg * 3.f)), both(m15));  // s_i / w_i
+            const F2 t = fma2<PK>(c, ce, o ? neg(ch) : ch);
+            const F2 ge = fma2<PK>(both(w), fma2<PK>(both(M.rho), s, t), wp3);
+            const F2 gn = fma2<PK>(both(omega_g), sub2<PK>(ge, gj), gj);
+            f[j] = fn.x;
+            f[j + 1] = fn.y;
+            g[j] = gn.x;
+            g[j + 1] = gn.y;
+        }
     }
     return phiu;
 }

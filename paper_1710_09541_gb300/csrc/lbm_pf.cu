@@ -15,7 +15,17 @@
 
 #include <cudaTypedefs.h>
 
+// Debug build (LBM_DEBUG_CHECKS = 1, the library liblbm_pf_debug.so): the
+// step checks every neighbour row and column and every shared-memory slot it
+// computes, records an out-of-range one as bit 4 of the error flag (the call
+// returns LBM_ERR_CUDA) and skips it, and poisons the tile's phi slots with
+// NaN before filling them.  It stands in for a sanitizer: the arithmetic is
+// the same, so results equal the release library's bit for bit.
+#ifndef LBM_DEBUG_CHECKS
+#define LBM_DEBUG_CHECKS 0
+#endif
 #include "lbm_kernels.cuh"
+#include "lbm_march.cuh"
 #include "lbm_pf.h"
 #include "lbm_store.cuh"
 
@@ -47,15 +57,6 @@ namespace {
 #endif
 #ifndef LBM_STEP_MINB
 #define LBM_STEP_MINB 0
-#endif
-// Debug build (LBM_DEBUG_CHECKS = 1, the library liblbm_pf_debug.so): the
-// step checks every neighbour row and column and every shared-memory slot it
-// computes, records an out-of-range one as bit 4 of the error flag (the call
-// returns LBM_ERR_CUDA) and skips it, and poisons the tile's phi slots with
-// NaN before filling them.  It stands in for a sanitizer: the arithmetic is
-// the same, so results equal the release library's bit for bit.
-#ifndef LBM_DEBUG_CHECKS
-#define LBM_DEBUG_CHECKS 0
 #endif
 #if LBM_DEBUG_CHECKS
 __device__ __forceinline__ bool nbr_in_range(const Nbr& q, int nx, int ny) {
@@ -133,8 +134,9 @@ __device__ __forceinline__ bool nbr_in_range(const Nbr& q, int nx, int ny) {
 template <int TX, int TY, bool FIELDS, int WALLS, int ST, bool CHK>
 __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __restrict__ fs,
                                           const float* __restrict__ gs, float* __restrict__ fd,
-                                          float* __restrict__ gd, float* __restrict__ phiu,
-                                          unsigned int* __restrict__ flag, double* __restrict__ out,
+                                          float* __restrict__ gd, const float* __restrict__ pus,
+                                          float* __restrict__ pud, unsigned int* __restrict__ flag,
+                                          double* __restrict__ out,
                                           int nx, int ny, Model m, int x0, int y0) {
     if (WALLS == 0) m.walls = 0;  // WALLS == 1 keeps the kind of top (wall or open)
     const int wfold = WALLS >= 0 ? WALLS : m.walls;  // y folding: wrap (0) or clamp
@@ -168,7 +170,7 @@ __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __
         }
 #endif
 #if LBM_EARLY_PHIU
-        if (!FIELDS) prev = make_float2(phiu[q.r0 + x], phiu[N32 + q.r0 + x]);
+        if (!FIELDS) prev = make_float2(pus[q.r0 + x], pus[N32 + q.r0 + x]);
 #endif
         pull18<ST, WALLS>(fs, gs, N32, q, f, g);
         sphi[ty + 1][tx + 1] = Pop<ST>::phi_of(f);
@@ -214,11 +216,11 @@ __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __
     if constexpr (CHK) bad = m.check_nonfinite && !isfinite(add(add(phi, M.ux), add(M.uy, M.p)));
 
 #if !LBM_EARLY_PHIU
-    const float2 prev = make_float2(phiu[n32], phiu[N32 + n32]);
+    const float2 prev = make_float2(pus[n32], pus[N32 + n32]);
 #endif
     const float2 now = collide_st<ST>(m, f, g, phi, st, M, prev);
-    phiu[n32] = now.x;
-    phiu[N32 + n32] = now.y;
+    pud[n32] = now.x;
+    pud[N32 + n32] = now.y;
     Pop<ST>::stfg(fd, gd, N32, n32, f, g, phi);
     if constexpr (CHK)
         if (bad) report_nonfinite(flag);
@@ -236,9 +238,9 @@ __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __
 template <int TX, int TY, int NPT, int WALLS, int ST, bool CHK>
 __device__ __forceinline__ void step_tile16(float (*sphi)[TX + 2], const void* __restrict__ fs,
                                             const void* __restrict__ gs, void* __restrict__ fd,
-                                            void* __restrict__ gd, float* __restrict__ phiu,
-                                            unsigned int* __restrict__ flag, int nx, int ny, Model m,
-                                            int x0, int y0) {
+                                            void* __restrict__ gd, const float* __restrict__ pus,
+                                            float* __restrict__ pud, unsigned int* __restrict__ flag,
+                                            int nx, int ny, Model m, int x0, int y0) {
     constexpr bool BR = (WALLS < 0) || LBM_WALL_BRANCH;
     constexpr int TH = TY * NPT;
     if (WALLS == 0) m.walls = 0;  // WALLS == 1 keeps the kind of top (wall or open)
@@ -272,7 +274,7 @@ __device__ __forceinline__ void step_tile16(float (*sphi)[TX + 2], const void* _
             }
 #endif
             n[j] = q.r0 + q.x;
-            prev[j] = make_float2(phiu[n[j]], phiu[N + n[j]]);
+            prev[j] = make_float2(pus[n[j]], pus[N + n[j]]);
             pull_words16<ST, BR, true>(fs, gs, N, q, w[j], f0[j], g0[j]);
             float h[9];
             codes_f<ST>(w[j], f0[j], h);
@@ -311,8 +313,8 @@ __device__ __forceinline__ void step_tile16(float (*sphi)[TX + 2], const void* _
         bool bad = false;
         if constexpr (CHK) bad = m.check_nonfinite && !isfinite(add(add(phi, M.ux), add(M.uy, M.p)));
         const float2 now = collide_code<Pop<ST>>(m, h, k, phi, st, M, prev[j]);
-        phiu[n[j]] = now.x;
-        phiu[N + n[j]] = now.y;
+        pud[n[j]] = now.x;
+        pud[N + n[j]] = now.y;
         Pop<ST>::stfg(fd, gd, N, n[j], h, k, phi, m.seed);
         if constexpr (CHK)
             if (bad) report_nonfinite(flag);
@@ -360,6 +362,7 @@ __device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* m, int x, int
                  "r"(x), "r"(y)
                  : "memory");
 }
+
 // tile (bx, by) of TX x TY nodes: the boxes start at column bx*TX (a multiple
 // of 32 elements, so 16-byte aligned) and at row by*TY - 1, clamped to 0 (the
 // top tile row then misses its wrapped halo row, which only costs a miss)
@@ -407,6 +410,21 @@ __device__ __forceinline__ void prefetch_tile(const void* fs, const void* gs, co
     }
 }
 
+// threads of each of the two sets of a march block, and resident threads per SM
+// (768: three blocks, 80 registers; see lbm_march.cuh for both sides)
+#ifndef LBM_MARCH_TW
+#define LBM_MARCH_TW 128
+#endif
+#ifndef LBM_MARCH_THREADS
+#define LBM_MARCH_THREADS 768
+#endif
+#ifndef LBM_MARCH_THREADS16
+#define LBM_MARCH_THREADS16 768
+#endif
+#ifndef LBM_MARCH_MIN_EFF
+#define LBM_MARCH_MIN_EFF 0.40
+#endif
+constexpr double MARCH_MIN_EFF = LBM_MARCH_MIN_EFF;
 // Resident blocks per SM each step kernel is compiled for (its register
 // budget), measured per instantiation with 32 x 4 tiles at 2048^2 (2400 x 600
 // for walls), MLUPS at 8 / 9 / 10 blocks:
@@ -435,8 +453,8 @@ __host__ __device__ constexpr int step_npt() {
 template <int TX, int TY, bool FIELDS, int WALLS, int ST, bool CHK = false>
 __global__ void __launch_bounds__(TX* TY, (step_minb<FIELDS, WALLS, ST, TX * TY>()))
     k_step(const float* __restrict__ fs, const float* __restrict__ gs, float* __restrict__ fd,
-           float* __restrict__ gd, float* __restrict__ phiu, unsigned int* __restrict__ flag,
-           double* __restrict__ out, int nx, int ny, Model m, int pf_ahead, int rev,
+           float* __restrict__ gd, const float* __restrict__ pus, float* __restrict__ pud,
+           unsigned int* __restrict__ flag, double* __restrict__ out, int nx, int ny, Model m, int pf_ahead, int rev,
            const __grid_constant__ PfMaps pm) {
     constexpr int NPT = step_npt<FIELDS, ST>();
     __shared__ float sphi[TY * NPT + 2][TX + 2];
@@ -459,17 +477,46 @@ __global__ void __launch_bounds__(TX* TY, (step_minb<FIELDS, WALLS, ST, TX * TY>
                 if (pm.on)
                     prefetch_tile_maps<TY * NPT, ST>(pm, px * TX, py);
                 else
-                    prefetch_tile<TX, TY * NPT, TX * TY, ST>(fs, gs, phiu, nx, ny,
+                    prefetch_tile<TX, TY * NPT, TX * TY, ST>(fs, gs, pus, nx, ny,
                                                              WALLS >= 0 ? WALLS : m.walls, px, py);
             }
         }
     }
     if constexpr (NPT > 1 || (!FIELDS && ST != ST_FP32))
-        step_tile16<TX, TY, NPT, WALLS, ST, CHK>(sphi, fs, gs, fd, gd, phiu, flag, nx, ny, m,
+        step_tile16<TX, TY, NPT, WALLS, ST, CHK>(sphi, fs, gs, fd, gd, pus, pud, flag, nx, ny, m,
                                                  bx * TX, by * TY * NPT);
     else
-        step_tile<TX, TY, FIELDS, WALLS, ST, CHK>(sphi, fs, gs, fd, gd, phiu, flag, out, nx, ny, m,
+        step_tile<TX, TY, FIELDS, WALLS, ST, CHK>(sphi, fs, gs, fd, gd, pus, pud, flag, out, nx, ny, m,
                                                   bx * TX, by * TY);
+}
+
+// Two steps per launch (lbm_march.cuh): block (strip, chunk) of a grid of
+// strips x chunks; odd chunks march downwards, and all of them the other way
+// when the step reads buffer 1 (par), so that neighbouring chunks meet at
+// their common rows and a launch starts on the rows the last one wrote last.
+struct MarchGrid {
+    int w, H;  // columns of a strip, rows of a chunk
+    int par;
+};
+constexpr int MARCH_TW = LBM_MARCH_TW;
+template <int ST>
+constexpr int march_minb() {
+    return (ST == ST_FP32 ? LBM_MARCH_THREADS : LBM_MARCH_THREADS16) / (2 * MARCH_TW);
+}
+template <int WALLS, int ST, bool CHK>
+__global__ void __launch_bounds__(2 * MARCH_TW, march_minb<ST>())
+    k_march(const __grid_constant__ MarchArgs A, const __grid_constant__ Model m, const MarchGrid G,
+            unsigned int seed2) {
+    extern __shared__ __align__(16) char march_smem[];
+    griddep_wait();
+    griddep_launch();
+    const int x0 = blockIdx.x * G.w, y0 = blockIdx.y * G.H;
+    const int y1 = min(y0 + G.H, A.ny), wlen = min(G.w, A.nx - x0), dir = (blockIdx.y + G.par) & 1 ? -1 : 1;
+    // (broadcast from lane 0, so that the compiler sees a warp-uniform branch)
+    if (__shfl_sync(0xffffffffu, (int)threadIdx.x, 0) < MARCH_TW)
+        march_block<1, MARCH_TW, WALLS, ST, CHK>(march_smem, A, m, x0, wlen, y0, y1, dir, seed2);
+    else
+        march_block<2, MARCH_TW, WALLS, ST, CHK>(march_smem, A, m, x0, wlen, y0, y1, dir, seed2);
 }
 
 // ---------------------------------------------------------------------------
@@ -533,7 +580,7 @@ __global__ void k_init(const double* __restrict__ in, void* __restrict__ fd,
 // Checkpoint out: canonical pre-collision state = the pulled populations.
 template <int ST>
 __global__ void k_state_out(const void* __restrict__ fs, const void* __restrict__ gs,
-                            const float* __restrict__ phiu, float* __restrict__ st, int nx,
+                            const float* phiu, float* st, int nx,
                             int ny, int walls) {
     const size_t N = (size_t)nx * ny;
     const int N32 = (int)N;
@@ -549,8 +596,10 @@ __global__ void k_state_out(const void* __restrict__ fs, const void* __restrict_
             st[i * N + n] = v[i];
             st[(9 + i) * N + n] = w[i];
         }
-        st[18 * N + n] = phiu[n];
-        st[19 * N + n] = phiu[N + n];
+        if (phiu != st + 18 * N) {  // the second (phi u) buffer is this place itself
+            st[18 * N + n] = phiu[n];
+            st[19 * N + n] = phiu[N + n];
+        }
     }
 }
 
@@ -694,7 +743,10 @@ struct lbm_handle {
     cudaStream_t stream = nullptr;
     float* f[2] = {nullptr, nullptr};
     float* g[2] = {nullptr, nullptr};
-    float* phiu = nullptr;
+    // (phi u) of the previous step, going with the population buffer of the
+    // same index; phiu[1] lives in the last 2 N floats of the staging buffer,
+    // where a checkpoint keeps it (no read-back writes there before reading it)
+    float* phiu[2] = {nullptr, nullptr};
     int cur = 0;
     void* staging = nullptr;   // host I/O staging: max(5 N doubles, 20 N floats)
     double* red_part = nullptr;  // RED_BLOCKS x 4 partials
@@ -706,6 +758,7 @@ struct lbm_handle {
     bool owns_memory = true;  // false: the device buffers live in a caller's workspace
     unsigned long long nstep = 0;  // steps since lbm_init: seeds the stochastic rounding
     PfMaps pm[2] = {};             // prefetch tensor maps of the step reading buffer 0 / 1
+    MarchGrid march = {0, 0, 0};   // strips and chunks of the two-step kernel (H = 0: not used)
     char err[512] = {0};
 };
 
@@ -786,7 +839,7 @@ static Model make_model(const lbm_params& p) {
 // not synchronise the whole device.
 static void release(lbm_handle* h) {
     if (!h->owns_memory) return;  // a caller's workspace stays the caller's
-    void* bufs[9] = {h->f[0], h->f[1], h->g[0], h->g[1], h->phiu, h->staging, h->red_part,
+    void* bufs[9] = {h->f[0], h->f[1], h->g[0], h->g[1], h->phiu[0], h->staging, h->red_part,
                      h->red_res, h->flag};
     for (void* b : bufs)
         if (b) cudaFreeAsync(b, h->stream);
@@ -844,11 +897,12 @@ static int grid1d(size_t N) {
 #define LBM_PDL 1
 #endif
 template <typename... Exp, typename... Act>
-static cudaError_t launch_dep(void (*k)(Exp...), dim3 grid, dim3 block, cudaStream_t s, Act&&... args) {
+static cudaError_t launch_dep(void (*k)(Exp...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              Act&&... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -867,7 +921,7 @@ static lbm_status launch_step(lbm_handle* h, bool fields, double* out) {
     const int th = st16 ? STEP_TY * LBM_NPT16 : STEP_TY;
     dim3 block(tw, STEP_TY);
     dim3 grid((h->nx + tw - 1) / tw, (h->ny + th - 1) / th);
-    using K = void (*)(const float*, const float*, float*, float*, float*, unsigned int*, double*,
+    using K = void (*)(const float*, const float*, float*, float*, const float*, float*, unsigned int*, double*,
                        int, int, Model, int, int, PfMaps);
     K k;
     // the steps of a handle that asked for non-finite checks test every node;
@@ -890,18 +944,84 @@ static lbm_status launch_step(lbm_handle* h, bool fields, double* out) {
     }
 #undef LBM_STEP_KERNEL
     if (fields)
-        k<<<grid, block, 0, h->stream>>>(h->f[c], h->g[c], nullptr, nullptr, h->phiu, h->flag, out,
-                                         h->nx, h->ny, h->model, 0, 0, PfMaps{});
+        k<<<grid, block, 0, h->stream>>>(h->f[c], h->g[c], nullptr, nullptr, h->phiu[c], nullptr, h->flag,
+                                         out, h->nx, h->ny, h->model, 0, 0, PfMaps{});
     else {
         // a distinct seed per step (the golden-ratio multiple of the step count)
         h->model.seed = (unsigned int)(++h->nstep) * 0x9e3779b9u;
-        LBM_CUDA(h, launch_dep(k, grid, block, h->stream, (const float*)h->f[c],
-                               (const float*)h->g[c], h->f[c ^ 1], h->g[c ^ 1], h->phiu, h->flag,
+        LBM_CUDA(h, launch_dep(k, grid, block, 0, h->stream, (const float*)h->f[c],
+                               (const float*)h->g[c], h->f[c ^ 1], h->g[c ^ 1],
+                               (const float*)h->phiu[c], h->phiu[c ^ 1], h->flag,
                                (double*)nullptr, h->nx, h->ny, h->model, h->pf_ahead,
                                LBM_ALTERNATE_ORDER ? c : 0, h->pm[c]));
     }
     LBM_CUDA(h, cudaGetLastError());
     if (!fields) h->cur ^= 1;
+    return LBM_OK;
+}
+
+// the kernel of the two-step march for a handle, and its shared memory
+using MarchKernel = void (*)(MarchArgs, Model, MarchGrid, unsigned int);
+template <int ST>
+static MarchKernel march_kernel_st(bool walls, bool chk) {
+    return walls ? (chk ? k_march<1, ST, true> : k_march<1, ST, false>)
+                 : (chk ? k_march<0, ST, true> : k_march<0, ST, false>);
+}
+static MarchKernel march_kernel(const lbm_params& p, size_t* smem) {
+    const bool walls = p.bc_y != LBM_BC_PERIODIC, chk = p.check_every > 0;
+    *smem = p.storage == LBM_STORE_FP32 ? MarchSmem<MARCH_TW, ST_FP32>::BYTES : MarchSmem<MARCH_TW, ST_FP16>::BYTES;
+    switch (p.storage) {
+        case LBM_STORE_FP16_SHIFTED: return march_kernel_st<ST_FP16>(walls, chk);
+        case LBM_STORE_BF16_SHIFTED: return march_kernel_st<ST_BF16>(walls, chk);
+        case LBM_STORE_BF16_SHIFTED_SR: return march_kernel_st<ST_BF16_SR>(walls, chk);
+        default: return march_kernel_st<ST_FP32>(walls, chk);
+    }
+}
+
+// Strips and chunks of a handle's two-step launches: one resident wave of
+// blocks.  A block computes TW columns for w of its own and about H + 7 rows'
+// time for H, so the march pays where w / TW * H / (H + 7) is high enough.
+static MarchGrid plan_march(int nx, int ny, const lbm_params& p, int sms) {
+    MarchGrid g = {0, 0, 0};
+    if (p.kernel == LBM_KERNEL_GENERIC || nx < 64 || ny < 16) return g;
+    const int most = MARCH_TW - 2 * MARCH_HALO;
+    const int strips = (nx + most - 1) / most;
+    g.w = (nx + strips - 1) / strips;
+    const int per_sm = p.storage == LBM_STORE_FP32 ? march_minb<ST_FP32>() : march_minb<ST_FP16>();
+    const int chunks = sms * per_sm / strips > 1 ? sms * per_sm / strips : 1;
+    g.H = (ny + chunks - 1) / chunks;
+    const double eff = (double)g.w / MARCH_TW * g.H / (g.H + 7);
+    if (eff < MARCH_MIN_EFF) g.H = 0;
+    return g;
+}
+
+// the planes of buffer c in the march's order (MarchArgs)
+static void march_planes(const lbm_handle* h, int c, char* p[20]) {
+    const bool st16 = h->prm.storage != LBM_STORE_FP32;
+    const int nf = 9, ng = st16 ? 1 : 9;
+    for (int i = 0; i < nf; ++i) p[i] = (char*)(h->f[c] + i * h->N);
+    for (int i = 0; i < ng; ++i) p[nf + i] = (char*)(h->g[c] + i * h->N);
+    for (int i = 0; i < 2; ++i) p[nf + ng + i] = (char*)(h->phiu[c] + i * h->N);
+}
+
+// two steps at once
+static lbm_status launch_march(lbm_handle* h) {
+    const int c = h->cur;
+    size_t smem;
+    const MarchKernel k = march_kernel(h->prm, &smem);
+    MarchGrid G = h->march;
+    G.par = c;
+    MarchArgs A{};
+    march_planes(h, c, (char**)A.s);
+    march_planes(h, c ^ 1, A.d);
+    A.flag = h->flag;
+    A.nx = h->nx;
+    A.ny = h->ny;
+    h->model.seed = (unsigned int)(++h->nstep) * 0x9e3779b9u;
+    const unsigned int seed2 = (unsigned int)(++h->nstep) * 0x9e3779b9u;
+    const dim3 grid((h->nx + G.w - 1) / G.w, (h->ny + G.H - 1) / G.H);
+    LBM_CUDA(h, launch_dep(k, grid, dim3(2 * MARCH_TW), smem, h->stream, A, h->model, G, seed2));
+    h->cur ^= 1;
     return LBM_OK;
 }
 
@@ -976,7 +1096,7 @@ static bool encode_maps16(const lbm_handle* h, int c, CUtensorMap m[4], int bx, 
                                static_cast<char*>((void*)h->f[c]) + 4 * N, 8, nx, ny, bx, by) &&
            encode_prefetch_map(&m[1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->f[c], 1, nx, ny, bx, by) &&
            encode_prefetch_map(&m[2], CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, h->g[c], 1, nx, ny, bx, by) &&
-           encode_prefetch_map(&m[3], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu, 2, nx, ny, bx, by);
+           encode_prefetch_map(&m[3], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu[c], 2, nx, ny, bx, by);
 }
 
 static void encode_pf_maps(lbm_handle* h) {
@@ -1005,7 +1125,7 @@ static void encode_pf_maps(lbm_handle* h) {
                                      tx, th + 2) &&
                  encode_prefetch_map(&pm.pop[1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->g[c], 9, nx, ny,
                                      tx, th + 2) &&
-                 encode_prefetch_map(&pm.phiu, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu, 2, nx, ny,
+                 encode_prefetch_map(&pm.phiu, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu[c], 2, nx, ny,
                                      tx, th + 2);
         }
         if (!ok) {
@@ -1029,7 +1149,7 @@ static lbm_status create_handle(int nx, int ny, const lbm_params* p, void* ws, l
     cudaError_t e = cudaGetDevice(&h->device);
     const Layout L = layout_of(nx, ny, p->storage);
     void** slot[9] = {(void**)&h->f[0], (void**)&h->f[1], (void**)&h->g[0], (void**)&h->g[1],
-                      (void**)&h->phiu, &h->staging,      (void**)&h->red_part, (void**)&h->red_res,
+                      (void**)&h->phiu[0], &h->staging,   (void**)&h->red_part, (void**)&h->red_res,
                       (void**)&h->flag};
     for (int k = 0; k < 9 && e == cudaSuccess; ++k) {
         if (ws)
@@ -1037,6 +1157,7 @@ static lbm_status create_handle(int nx, int ny, const lbm_params* p, void* ws, l
         else
             e = cudaMallocAsync(slot[k], L.size[k], h->stream);
     }
+    h->phiu[1] = (float*)h->staging + 18 * h->N;
     if (e == cudaSuccess) e = cudaMemsetAsync(h->flag, 0, sizeof(unsigned int), h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     int sms = 0;
@@ -1060,6 +1181,12 @@ static lbm_status create_handle(int nx, int ny, const lbm_params* p, void* ws, l
             // no maps after all: the per-thread requests' own threshold
             if (st16 && !h->pm[0].on && bytes * 10.0 < (double)LBM_PREFETCH16_L2X10 * l2) h->pf_ahead = 0;
         }
+    }
+    h->march = plan_march(nx, ny, *p, sms);
+    if (e == cudaSuccess && h->march.H > 0) {
+        size_t smem;
+        const MarchKernel k = march_kernel(*p, &smem);
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
     if (e != cudaSuccess) {
         fprintf(stderr, "lbm_create: %s\n", cudaGetErrorString(e));
@@ -1157,7 +1284,7 @@ lbm_status lbm_init(lbm_handle* h, const double* phi0, const double* ux0, const 
     auto kinit = h->prm.storage == LBM_STORE_FP16_SHIFTED ? k_init<ST_FP16>
                  : is_bf16(h->prm.storage)                ? k_init<ST_BF16>
                                                           : k_init<ST_FP32>;
-    kinit<<<grid1d(h->N), 256, 0, h->stream>>>(in, h->f[0], h->g[0], h->phiu, h->nx, h->ny,
+    kinit<<<grid1d(h->N), 256, 0, h->stream>>>(in, h->f[0], h->g[0], h->phiu[0], h->nx, h->ny,
                                                  h->model);
     LBM_CUDA(h, cudaGetLastError());
     LBM_CUDA(h, cudaMemsetAsync(h->flag, 0, sizeof(unsigned int), h->stream));
@@ -1173,10 +1300,14 @@ lbm_status lbm_step(lbm_handle* h, int nsteps) {
     if (nsteps < 0) return fail(h, LBM_ERR_INVALID, "lbm_step: nsteps < 0");
     if (!h->inited) return fail(h, LBM_ERR_STATE, "lbm_step before lbm_init");
     LBM_CUDA(h, cudaSetDevice(h->device));
-    for (int s = 0; s < nsteps; ++s) {
-        lbm_status st = launch_step(h, false, nullptr);
+    for (int s = 0; s < nsteps;) {
+        // two steps at once, unless a check falls between them
+        const bool two = h->march.H > 0 && nsteps - s >= 2 &&
+                         (h->prm.check_every == 0 || h->prm.check_every - h->since_check >= 2);
+        lbm_status st = two ? launch_march(h) : launch_step(h, false, nullptr);
         if (st != LBM_OK) return st;
-        if (h->prm.check_every > 0 && ++h->since_check >= h->prm.check_every) {
+        s += two ? 2 : 1;
+        if (h->prm.check_every > 0 && (h->since_check += two ? 2 : 1) >= h->prm.check_every) {
             st = check_flag(h);
             if (st != LBM_OK) return st;
         }
@@ -1212,7 +1343,7 @@ lbm_status lbm_get_state(lbm_handle* h, void* host_buf, size_t bytes) {
     auto kout = h->prm.storage == LBM_STORE_FP16_SHIFTED ? k_state_out<ST_FP16>
                 : is_bf16(h->prm.storage)                ? k_state_out<ST_BF16>
                                                           : k_state_out<ST_FP32>;
-    kout<<<grid1d(h->N), 256, 0, h->stream>>>(h->f[h->cur], h->g[h->cur], h->phiu, st,
+    kout<<<grid1d(h->N), 256, 0, h->stream>>>(h->f[h->cur], h->g[h->cur], h->phiu[h->cur], st,
                                                       h->nx, h->ny, h->model.walls);
     LBM_CUDA(h, cudaGetLastError());
     LBM_CUDA(h, cudaMemcpyAsync(host_buf, st, bytes, cudaMemcpyDeviceToHost, h->stream));
@@ -1232,7 +1363,7 @@ lbm_status lbm_set_state(lbm_handle* h, const void* host_buf, size_t bytes) {
     auto kin = h->prm.storage == LBM_STORE_FP16_SHIFTED ? k_state_in<ST_FP16>
                : is_bf16(h->prm.storage)                ? k_state_in<ST_BF16>
                                                          : k_state_in<ST_FP32>;
-    kin<<<grid1d(h->N), 256, 0, h->stream>>>(st, h->f[0], h->g[0], h->phiu, h->nx,
+    kin<<<grid1d(h->N), 256, 0, h->stream>>>(st, h->f[0], h->g[0], h->phiu[0], h->nx,
                                                      h->ny, h->model.walls);
     LBM_CUDA(h, cudaGetLastError());
     LBM_CUDA(h, cudaMemsetAsync(h->flag, 0, sizeof(unsigned int), h->stream));
@@ -1439,7 +1570,7 @@ namespace {
 struct CaseDesc {
     float* f[2];
     float* g[2];
-    float* phiu;
+    float* phiu[2];
     unsigned int* flag;
     int nx, ny;
     int cur;   // buffer holding the current state when the batch parity is 0
@@ -1455,8 +1586,6 @@ constexpr int BATCH_PF_BOX_X = 32, BATCH_PF_BOX_Y = 10;
 struct BatchTable {
     const CUtensorMap* maps;  // 16-bit prefetch maps in device memory (nullptr: per-thread requests)
     int ncases;
-    int tiles_x[BATCH_MAX_CASES];
-    int tile0[BATCH_MAX_CASES + 1];  // first tile of each case; tile0[ncases] = total
     CaseDesc c[BATCH_MAX_CASES];
 };
 static_assert(sizeof(BatchTable) <= 32000, "kernel parameters are limited to 32 KB");
@@ -1524,7 +1653,7 @@ __global__ void __launch_bounds__(TX* TY, (ST == ST_FP32 ? LBM_BATCH_THREADS : L
                     tma_prefetch_3d(mp, x, y, 0);
             }
         } else {
-            prefetch_tile<TX, TH, TX * TY, ST>(pc.f[pcur], pc.g[pcur], pc.phiu, pc.nx, pc.ny, WALLS,
+            prefetch_tile<TX, TH, TX * TY, ST>(pc.f[pcur], pc.g[pcur], pc.phiu[pcur], pc.nx, pc.ny, WALLS,
                                                pe.y & 0xffff, pe.y >> 16);
         }
     }
@@ -1541,12 +1670,12 @@ __global__ void __launch_bounds__(TX* TY, (ST == ST_FP32 ? LBM_BATCH_THREADS : L
     const CaseDesc& cd = T.c[e.x];
     const int c = (cd.cur + parity) & 1;
     if constexpr (ST == ST_FP32) {
-        step_tile<TX, TY, false, WALLS, ST, CHK>(sphi, cd.f[c], cd.g[c], cd.f[c ^ 1], cd.g[c ^ 1], cd.phiu,
-                                            cd.flag, nullptr, cd.nx, cd.ny, cd.m, (e.y & 0xffff) * TX,
+        step_tile<TX, TY, false, WALLS, ST, CHK>(sphi, cd.f[c], cd.g[c], cd.f[c ^ 1], cd.g[c ^ 1],
+                                                 cd.phiu[c], cd.phiu[c ^ 1], cd.flag, nullptr, cd.nx, cd.ny, cd.m, (e.y & 0xffff) * TX,
                                             (e.y >> 16) * TY);
     } else {
         step_tile16<TX, TY, LBM_NPT16_BATCH, WALLS, ST, CHK>(
-            sphi, cd.f[c], cd.g[c], cd.f[c ^ 1], cd.g[c ^ 1], cd.phiu, cd.flag, cd.nx, cd.ny, cd.m,
+            sphi, cd.f[c], cd.g[c], cd.f[c ^ 1], cd.g[c ^ 1], cd.phiu[c], cd.phiu[c ^ 1], cd.flag, cd.nx, cd.ny, cd.m,
             (e.y & 0xffff) * TX, (e.y >> 16) * TY * LBM_NPT16_BATCH);
     }
 }
@@ -1617,6 +1746,7 @@ struct lbm_batch {
     cudaEvent_t t0 = nullptr, t1 = nullptr;
     BatchTable* table = nullptr;  // [class][shape], host side, passed by value
     int2* d_tiles[BATCH_NCLASS * BATCH_NCAND] = {};  // tile lists on the device, [class][shape]
+    int tiles[BATCH_NCLASS * BATCH_NCAND] = {};      // and their lengths
     bool check = false;                 // some case asks for non-finite checks (check_every > 0)
     int* d_slot[BATCH_NCLASS] = {};     // per class: the batch index of each class slot
     unsigned int* d_flags = nullptr;    // gathered flags, one per case
@@ -1690,7 +1820,7 @@ static lbm_status batch_launch(lbm_batch* b, int cls, int cand, int parity) {
     const BatchTable& T = b->tab(cls, cand);
     // programmatic dependent launch, as for the single-case steps (also inside
     // the captured graph, where it becomes a programmatic edge)
-    LBM_BCUDA(b, launch_dep(k, dim3(T.tile0[T.ncases]), dim3(BATCH_TX[cand], BATCH_TY[cand]),
+    LBM_BCUDA(b, launch_dep(k, dim3(b->tiles[cls * BATCH_NCAND + cand]), dim3(BATCH_TX[cand], BATCH_TY[cand]), 0,
                             b->bs[cls], T, (const int2*)b->d_tiles[cls * BATCH_NCAND + cand], parity,
                             b->pf_ahead));
     return LBM_OK;
@@ -1881,27 +2011,26 @@ lbm_status lbm_batch_create(int ncases, lbm_handle* const* cases, lbm_batch** ou
                 d.f[1] = h->f[1];
                 d.g[0] = h->g[0];
                 d.g[1] = h->g[1];
-                d.phiu = h->phiu;
+                d.phiu[0] = h->phiu[0];
+                d.phiu[1] = h->phiu[1];
                 d.flag = h->flag;
                 d.nx = h->nx;
                 d.ny = h->ny;
                 d.cur = h->cur;
                 d.map0 = -1;
                 d.m = h->model;
-                T.tiles_x[j] = (h->nx + BATCH_TX[k] - 1) / BATCH_TX[k];
-                T.tile0[j] = (int)tiles;
-                tiles += (long long)T.tiles_x[j] * ((h->ny + th - 1) / th);
+                tiles += (long long)((h->nx + BATCH_TX[k] - 1) / BATCH_TX[k]) * ((h->ny + th - 1) / th);
             }
             if (tiles >= (1LL << 31) - 1) {
                 bfail(b, LBM_ERR_INVALID, "batch too large for one launch");
                 return bad(LBM_ERR_INVALID);
             }
-            T.tile0[T.ncases] = (int)tiles;
+            b->tiles[cls * BATCH_NCAND + k] = (int)tiles;
             // the tile list: (case, tile row << 16 | tile column), case-major
             std::vector<int2> list((size_t)tiles);
             size_t n = 0;
             for (int j = 0; j < T.ncases; ++j) {
-                const int tx = T.tiles_x[j], ty = (T.c[j].ny + th - 1) / th;
+                const int tx = (T.c[j].nx + BATCH_TX[k] - 1) / BATCH_TX[k], ty = (T.c[j].ny + th - 1) / th;
                 if (tx > 0xffff || ty > 0x7fff) {
                     bfail(b, LBM_ERR_INVALID, "a case has more than 65535 x 32767 tiles");
                     return bad(LBM_ERR_INVALID);

@@ -97,8 +97,14 @@ struct Pop<ST_FP32> {
     // the pulled f (Eq. 12), the moments of g (Eq. 22), the pulled values as
     // populations, and the rest population f_0 that makes the stored
     // populations of an initial state sum to phi
-    __device__ static float phi_of(const float f[9]) { return sum9(f); }
-    __device__ static GMom gmom(const float g[9]) { return gmoments(g); }
+    template <bool PK = false>
+    __device__ static float phi_of(const float f[9]) {
+        return sum9<PK>(f);
+    }
+    template <bool PK = false>
+    __device__ static GMom gmom(const float g[9]) {
+        return gmoments<PK>(g);
+    }
     __device__ static void canon(float*, float*) {}
     __device__ static float init_rest(float phi, const float fe[9]) { return sub(phi, sum8(fe)); }
     // population planes, and the address of entry idx of plane k (prefetches)
@@ -215,20 +221,27 @@ struct Shifted16 {
     // f_0 + s8 gives phi back exactly (f_0 = phi - s8 is exact by Sterbenz's
     // lemma) and their roundings cannot drift sum phi in one direction
     static constexpr float HALF_MOVING = 0.5f * (4.f * w_of(1) + 4.f * w_of(5));
+    template <bool PK = false>
     __device__ static float s8(const float h[9]) {
-        const float a = add(add(h[1], h[3]), add(h[2], h[4]));
-        const float d = add(add(h[5], h[7]), add(h[6], h[8]));
-        return fma_rn(w_of(1), a, fma_rn(w_of(5), d, HALF_MOVING));
+        const F2 a = add2<PK>(dirs(h, 1), dirs(h, 3)), d = add2<PK>(dirs(h, 5), dirs(h, 7));
+        return fma_rn(w_of(1), add(a.x, a.y), fma_rn(w_of(5), add(d.x, d.y), HALF_MOVING));
     }
-    __device__ static float phi_of(const float h[9]) { return add(h[0], s8(h)); }
+    template <bool PK = false>
+    __device__ static float phi_of(const float h[9]) {
+        return add(h[0], s8<PK>(h));
+    }
     // the moments of g (Eq. 22) from the codes k_i
+    template <bool PK = false>
     __device__ static GMom gmom(const float k[9]) {
         constexpr float a1 = w_of(1) / GS, a5 = w_of(5) / GS;  // exact: GS is a power of 2
         GMom o;
-        o.mx = fma_rn(a1, sub(k[1], k[3]), mul(a5, add(sub(k[5], k[6]), sub(k[8], k[7]))));
-        o.my = fma_rn(a1, sub(k[2], k[4]), mul(a5, add(sub(k[5], k[8]), sub(k[6], k[7]))));
-        o.snz = fma_rn(a1, add(add(k[1], k[3]), add(k[2], k[4])),
-                       mul(a5, add(add(k[5], k[7]), add(k[6], k[8]))));
+        const F2 d = sub2<PK>(dirs(k, 1), dirs(k, 3));
+        const F2 dd{add(sub(k[5], k[6]), sub(k[8], k[7])), add(sub(k[5], k[8]), sub(k[6], k[7]))};
+        const F2 mv = fma2<PK>(both(a1), d, mul2<PK>(both(a5), dd));
+        o.mx = mv.x;
+        o.my = mv.y;
+        const F2 a = add2<PK>(dirs(k, 1), dirs(k, 3)), b = add2<PK>(dirs(k, 5), dirs(k, 7));
+        o.snz = fma_rn(a1, add(a.x, a.y), mul(a5, add(b.x, b.y)));
         return o;
     }
     // codes -> populations (checkpoint read-out)
@@ -245,16 +258,16 @@ struct Shifted16 {
         for (int i = 1; i < 9; ++i) h[i] = C::to_f(enc_f(i, fe[i]));
         return sub(phi, s8(h));
     }
-    // store the post-collision codes of node idx: h_i | k_i << 16 per moving
-    // direction, k_0, and f_0 as the remainder phi - s8(stored codes); seed
-    // (SR only) is the step's seed of the dithers
-    __device__ static void stfg(void* fb, void* gb, int N, int idx, const float h[9],
-                                const float k[9], float phi, unsigned int seed = 0) {
+    // the post-collision codes of node idx as stored: w[i] = h_i | k_i << 16 per
+    // moving direction, k_0, and f_0 as the remainder phi - s8(stored codes);
+    // seed (SR only) is the step's seed of the dithers
+    template <bool PK = false>
+    __device__ static void encode(const float h[9], const float k[9], float phi, unsigned int idx,
+                                  unsigned int seed, unsigned int w[9], float& f0, unsigned short& k0) {
         static_assert(!SR || C::GS == 1.f, "stochastic rounding is a BF16 format");
-        unsigned int* P = pw(fb, N);
         float d[9];
         if constexpr (SR) {
-            const unsigned int base = lowbias32((unsigned int)idx ^ seed);
+            const unsigned int base = lowbias32(idx ^ seed);
 #pragma unroll
             for (int i = 1; i < 9; i += 2) {
                 // directions i and i + 1 take the upper and lower halves of
@@ -263,26 +276,34 @@ struct Shifted16 {
                 const unsigned int r = (base + (unsigned int)(i >> 1) * 0x9e3779b9u) * 0x85ebca6bu;
                 const unsigned int kk = bf16x2_sr(k[i], k[i + 1], r);
                 const unsigned int hh = C::pack(h[i], h[i + 1]);
-                const unsigned int wi = __byte_perm(hh, kk, 0x7610);
-                const unsigned int wj = __byte_perm(hh, kk, 0x5432);
-                P[(i - 1) * N + idx] = wi;
-                P[i * N + idx] = wj;
-                d[i] = C::to_f(lo(wi));
-                d[i + 1] = C::to_f(lo(wj));
+                w[i] = __byte_perm(hh, kk, 0x7610);
+                w[i + 1] = __byte_perm(hh, kk, 0x5432);
+                d[i] = C::to_f(lo(w[i]));
+                d[i + 1] = C::to_f(lo(w[i + 1]));
             }
-            static_cast<float*>(fb)[idx] = sub(phi, s8(d));
-            static_cast<unsigned short*>(gb)[idx] =
-                (unsigned short)(bf16x2_sr(k[0], 0.f, (base + 4u * 0x9e3779b9u) * 0x85ebca6bu) >> 16);
+            k0 = (unsigned short)(bf16x2_sr(k[0], 0.f, (base + 4u * 0x9e3779b9u) * 0x85ebca6bu) >> 16);
         } else {
 #pragma unroll
             for (int i = 1; i < 9; ++i) {
-                const unsigned int w = C::pack(h[i], k[i]);
-                P[(i - 1) * N + idx] = w;
-                d[i] = C::to_f(lo(w));
+                w[i] = C::pack(h[i], k[i]);
+                d[i] = C::to_f(lo(w[i]));
             }
-            static_cast<float*>(fb)[idx] = sub(phi, s8(d));
-            static_cast<unsigned short*>(gb)[idx] = C::from_f(k[0]);
+            k0 = C::from_f(k[0]);
         }
+        f0 = sub(phi, s8<PK>(d));
+    }
+    // store the post-collision codes of node idx
+    __device__ static void stfg(void* fb, void* gb, int N, int idx, const float h[9],
+                                const float k[9], float phi, unsigned int seed = 0) {
+        unsigned int* P = pw(fb, N);
+        unsigned int w[9];
+        float f0;
+        unsigned short k0;
+        encode(h, k, phi, (unsigned int)idx, seed, w, f0, k0);
+#pragma unroll
+        for (int i = 1; i < 9; ++i) P[(i - 1) * N + idx] = w[i];
+        static_cast<float*>(fb)[idx] = f0;
+        static_cast<unsigned short*>(gb)[idx] = k0;
     }
     // one entry (checkpoint and initial-state permutations)
     __device__ static void putf(void* fb, int N, int i, int idx, float v) {
@@ -325,18 +346,17 @@ struct Pop<ST_BF16_SR> : Shifted16<__nv_bfloat16, true> {};
 // i > 0, GS (rho s_0 / w_0 + 3 p (w_0 - 1) / w_0) for i = 0, with s_i / w_i =
 // 3 c_i.u + 4.5 (c_i.u)^2 - 1.5 |u|^2.  f_0 is not collided: the store writes
 // it as the remainder.  Returns (phi ux, phi uy).
-template <class P>
+template <class P, bool PK = false>
 __device__ __forceinline__ float2 collide_code(const Model& m, float h[9], float k[9], float phi,
                                                const Stencil& st, const Macro& M, float2 phiu_prev) {
     constexpr float GS = P::GS;
     const float ux = M.ux, uy = M.uy;
     const float nu = viscosity(m, phi, M.inv_rho);                     // Eqs. 23-26
     const float omega_g = rcp_approx(fma_rn(3.f, nu, 0.5f));
-    float cu[9];
-    cdot9(ux, uy, cu);
-    const float2 phiu = make_float2(mul(phi, ux), mul(phi, uy));
-    const float Dx = sub(phiu.x, phiu_prev.x);                          // d_t(phi u), Eq. 11
-    const float Dy = sub(phiu.y, phiu_prev.y);
+    const F2 pu = mul2<PK>(both(phi), F2{ux, uy});
+    const F2 D = sub2<PK>(pu, F2{phiu_prev.x, phiu_prev.y});            // d_t(phi u), Eq. 11
+    const float2 phiu = make_float2(pu.x, pu.y);
+    const float Dx = D.x, Dy = D.y;
     const float lam = mul(mul(m.four_over_W, phi), sub(1.f, phi));      // Eq. 3
     const float phm = sub(phi, 0.5f);
     float nx_ = 0.f, ny_ = 0.f;
@@ -348,7 +368,8 @@ __device__ __forceinline__ float2 collide_code(const Model& m, float h[9], float
             ny_ = mul(st.gy, inv);
         }
     } else {  // Eq. 29: C = sum c_i (f_i - f_i^eq) + d_t(phi u)/2, n = -C/|C|
-        float ne[9];  // (f_i - f_i^eq) / w_i
+        float ne[9], cu[9];  // (f_i - f_i^eq) / w_i
+        cdot9(ux, uy, cu);
 #pragma unroll
         for (int i = 1; i < 9; ++i) ne[i] = sub(h[i], fma_rn(3.f, cu[i], phm));
         const float Cx = add(mul(0.5f, Dx), fma_rn(w_of(1), sub(ne[1], ne[3]),
@@ -362,24 +383,30 @@ __device__ __forceinline__ float2 collide_code(const Model& m, float h[9], float
             ny_ = -mul(Cy, inv);
         }
     }
+    // c_i . v of directions i, i + 1 (i = 1: vx, vy; i = 5: vx + vy, vy - vx);
+    // directions i + 2, i + 3 take the other sign
+    auto cdot = [](int i, F2 v) { return i == 1 ? v : F2{add(v.x, v.y), sub(v.y, v.x)}; };
     // Allen-Cahn, Eqs. 8, 9, 11 (first, so c_i . V is dead before the g terms)
     {
-        const float l3 = mul(lam, 1.f / 3.f);
-        float cv[9];
-        cdot9(fma_rn(m.tau_f_mh, fma_rn(l3, nx_, Dx), phiu.x),
-              fma_rn(m.tau_f_mh, fma_rn(l3, ny_, Dy), phiu.y), cv);   // c_i . V
+        const F2 V = fma2<PK>(both(m.tau_f_mh), fma2<PK>(both(mul(lam, 1.f / 3.f)), F2{nx_, ny_}, D), pu);
 #pragma unroll
-        for (int i = 1; i < 9; ++i) {
-            const float he = fma_rn(3.f, cv[i], phm);
-            h[i] = fma_rn(m.inv_tau_f, sub(he, h[i]), h[i]);
+        for (int i = 1; i < 9; i += 4) {
+            const F2 cv = cdot(i, V);
+#pragma unroll
+            for (int o = 0; o < 2; ++o) {
+                const int j = i + 2 * o;
+                const F2 hj = dirs(h, j);
+                const F2 he = fma2<PK>(both(o ? -3.f : 3.f), cv, both(phm));
+                const F2 hn = fma2<PK>(both(m.inv_tau_f), sub2<PK>(he, hj), hj);
+                h[j] = hn.x;
+                h[j + 1] = hn.y;
+            }
         }
     }
     // Navier-Stokes, Eqs. 15-17, 20
-    float ch[9], ce[9];
-    const float nu9 = mul(9.f * GS, nu);                          // GS scalings are exact
-    cdot9(mul(nu9, M.Fx), mul(nu9, M.Fy), ch);                    // GS c_i . 3 nu 3F
-    const float e9 = mul(nu9, m.drho);
-    cdot9(mul(e9, st.gx), mul(e9, st.gy), ce);                    // GS c_i . 3 nu 3 (rho_l - rho_g) grad phi
+    const float nu9 = mul(9.f * GS, nu);                              // GS scalings are exact
+    const F2 hv = mul2<PK>(both(nu9), F2{M.Fx, M.Fy});                // GS c_i . 3 nu 3F
+    const F2 ev = mul2<PK>(both(mul(nu9, m.drho)), F2{st.gx, st.gy});  // GS c_i . 3 nu 3 (rho_l - rho_g) grad phi
     const float p3 = mul(3.f * GS, M.p);
     const float rho = mul(GS, M.rho);
     const float m15 = mul(-1.5f, M.usq);
@@ -393,26 +420,29 @@ __device__ __forceinline__ float2 collide_code(const Model& m, float h[9], float
     // 3F with opposite signs: A + B and A - B.
     const float rho3 = mul(3.f, rho);
 #pragma unroll
-    for (int i = 1; i < 9; ++i) {
-        if (i == 3 || i == 4 || i == 7 || i == 8) continue;  // done with its opposite
-        const int o = opp_of(i);
-        const float c = cu[i];
-        const float A = fma_rn(rho, fma_rn(mul(4.5f, c), c, m15), fma_rn(c, ce[i], p3));
-        const float B = fma_rn(rho3, c, ch[i]);
-        k[i] = fma_rn(omega_g, sub(add(A, B), k[i]), k[i]);
-        k[o] = fma_rn(omega_g, sub(sub(A, B), k[o]), k[o]);
+    for (int i = 1; i < 9; i += 4) {
+        const F2 c = cdot(i, F2{ux, uy}), kp = dirs(k, i), km = dirs(k, i + 2);
+        const F2 A = fma2<PK>(both(rho), fma2<PK>(mul2<PK>(both(4.5f), c), c, both(m15)),
+                              fma2<PK>(c, cdot(i, ev), both(p3)));
+        const F2 B = fma2<PK>(both(rho3), c, cdot(i, hv));
+        const F2 np = fma2<PK>(both(omega_g), sub2<PK>(add2<PK>(A, B), kp), kp);
+        const F2 nm = fma2<PK>(both(omega_g), sub2<PK>(sub2<PK>(A, B), km), km);
+        k[i] = np.x;
+        k[i + 1] = np.y;
+        k[i + 2] = nm.x;
+        k[i + 3] = nm.y;
     }
     return phiu;
 }
 
 // The collision of the storage format ST: on populations (FP32) or on codes.
-template <int ST>
+template <int ST, bool PK = false>
 __device__ __forceinline__ float2 collide_st(const Model& m, float f[9], float g[9], float phi,
                                              const Stencil& st, const Macro& M, float2 prev) {
     if constexpr (ST == ST_FP32)
-        return collide(m, f, g, phi, st, M, prev);
+        return collide<PK>(m, f, g, phi, st, M, prev);
     else
-        return collide_code<Pop<ST>>(m, f, g, phi, st, M, prev);
+        return collide_code<Pop<ST>, PK>(m, f, g, phi, st, M, prev);
 }
 
 // Pull (stream) node q through a 16-bit storage format: the nine loads (f_0
