@@ -120,7 +120,7 @@ struct MarchRow {  // 16-bit formats: the code words as stored
     __device__ __forceinline__ void pull_ring_phi(const char* ring, const PullOff& o, bool lo, bool hi) {
         f0 = sh<float>(ring + o.cc);
         w[0] = 0u;
-        pull_dirs<WALLS, false>([&](int i, unsigned int off) { return sh<unsigned int>(ring + off + i * LP); }, o,
+        pull_dirs<WALLS, false>([&](int i, unsigned int off) { return sh<unsigned int>(ring + (int)off + i * LP); }, o,
                                 lo, hi, w);
     }
     template <bool WALLS, int LP>
@@ -180,12 +180,12 @@ struct MarchRow<ST_FP32> {
     }
     template <bool WALLS, int LP>
     __device__ __forceinline__ void pull_ring_phi(const char* ring, const PullOff& o, bool lo, bool hi) {
-        pull_dirs<WALLS, true>([&](int i, unsigned int off) { return sh<float>(ring + off + i * LP); }, o, lo, hi, f);
+        pull_dirs<WALLS, true>([&](int i, unsigned int off) { return sh<float>(ring + (int)off + i * LP); }, o, lo, hi, f);
     }
     template <bool WALLS, int LP>
     __device__ __forceinline__ void pull_ring(const char* ring, const PullOff& o, bool lo, bool hi) {
         pull_ring_phi<WALLS, LP>(ring, o, lo, hi);
-        pull_dirs<WALLS, true>([&](int i, unsigned int off) { return sh<float>(ring + off + (9 + i) * LP); }, o, lo,
+        pull_dirs<WALLS, true>([&](int i, unsigned int off) { return sh<float>(ring + (int)off + (9 + i) * LP); }, o, lo,
                                hi, g);
         prev = make_float2(sh<float>(ring + o.cc + 18 * LP), sh<float>(ring + o.cc + 19 * LP));
     }

@@ -28,6 +28,7 @@
 #include "lbm_march.cuh"
 #include "lbm_pf.h"
 #include "lbm_store.cuh"
+#include "lbm_tile.cuh"
 
 using namespace lbmpf;
 
@@ -519,6 +520,22 @@ __global__ void __launch_bounds__(2 * MARCH_TW, march_minb<ST>())
         march_block<2, MARCH_TW, WALLS, ST, CHK>(march_smem, A, m, x0, wlen, y0, y1, dir, seed2);
 }
 
+// S steps per launch of a small grid (lbm_tile.cuh): block (bx, by) owns tile
+// (bx, by) of w x h nodes; nstep: steps taken so far (seeds the dithers).
+struct TileGrid {
+    int w, h, S;
+};
+template <int WALLS, int ST, bool CHK>
+__global__ void __launch_bounds__(TILE_THREADS)
+    k_tile(const __grid_constant__ MarchArgs A, const __grid_constant__ Model m, const TileGrid G,
+           unsigned int nstep) {
+    __shared__ __align__(16) char smem[TileSmem<ST>::BYTES];
+    griddep_wait();
+    griddep_launch();
+    const int x0 = blockIdx.x * G.w, y0 = blockIdx.y * G.h;
+    tile_block<WALLS, ST, CHK>(smem, A, m, x0, y0, min(G.w, A.nx - x0), min(G.h, A.ny - y0), G.S, nstep);
+}
+
 // ---------------------------------------------------------------------------
 // Initial state.  The canonical (pre-collision) state is f_i = f_i^eq(phi0,u0)
 // (Eq. 9) and g_i = g_i^eq(p0, rho(phi0), u0) (Eqs. 13, 16, 17).  The pull
@@ -758,6 +775,7 @@ struct lbm_handle {
     bool owns_memory = true;  // false: the device buffers live in a caller's workspace
     unsigned long long nstep = 0;  // steps since lbm_init: seeds the stochastic rounding
     PfMaps pm[2] = {};             // prefetch tensor maps of the step reading buffer 0 / 1
+    TileGrid tile = {0, 0, 0};     // tiles of the several-step kernel (S = 0: not used)
     MarchGrid march = {0, 0, 0};   // strips and chunks of the two-step kernel (H = 0: not used)
     char err[512] = {0};
 };
@@ -1004,6 +1022,76 @@ static void march_planes(const lbm_handle* h, int c, char* p[20]) {
     for (int i = 0; i < 2; ++i) p[nf + ng + i] = (char*)(h->phiu[c] + i * h->N);
 }
 
+static MarchArgs march_args(const lbm_handle* h) {
+    MarchArgs A{};
+    march_planes(h, h->cur, (char**)A.s);
+    march_planes(h, h->cur ^ 1, A.d);
+    A.flag = h->flag;
+    A.nx = h->nx;
+    A.ny = h->ny;
+    return A;
+}
+
+using TileKernel = void (*)(MarchArgs, Model, TileGrid, unsigned int);
+template <int ST>
+static TileKernel tile_kernel_st(bool walls, bool chk) {
+    return walls ? (chk ? k_tile<1, ST, true> : k_tile<1, ST, false>)
+                 : (chk ? k_tile<0, ST, true> : k_tile<0, ST, false>);
+}
+static TileKernel tile_kernel(const lbm_params& p) {
+    const bool walls = p.bc_y != LBM_BC_PERIODIC, chk = p.check_every > 0;
+    switch (p.storage) {
+        case LBM_STORE_FP16_SHIFTED: return tile_kernel_st<ST_FP16>(walls, chk);
+        case LBM_STORE_BF16_SHIFTED: return tile_kernel_st<ST_BF16>(walls, chk);
+        case LBM_STORE_BF16_SHIFTED_SR: return tile_kernel_st<ST_BF16_SR>(walls, chk);
+        default: return tile_kernel_st<ST_FP32>(walls, chk);
+    }
+}
+
+// Tiles and steps per launch of a small grid, by the time they should take.
+// Measured on GB300 (FP32, a block per SM), a launch of S steps takes about
+// 1.78 us + 2.8 ns per node of the regions its steps compute, that once per
+// wave of blocks (8 x 8 tiles on 64^2: S = 2 / 3 / 4 2.59 / 3.49 / 4.84 us;
+// 16 x 8 tiles on 128^2, S = 3: 4.19 us, 26 x 10 on 256^2, S = 2: 6.59 us); the
+// 16-bit formats take 3 to 8% less.  A one-step launch takes about 2.45 us +
+// 15 ns per 1000 nodes (FP32: 64^2 2.56, 256^2 3.36, 384^2 5.13) or 3 us + 9 ns
+// (16 bits: 3.18, 3.70, 4.31).  us per step, one-step kernel -> tiles: FP32 64^2
+// 2.56 -> 1.06, 8 x 256 walled 2.92 -> 1.01, 128^2 2.60 -> 1.40, 200^2 3.53 ->
+// 2.69; FP16 64^2 3.18 -> 1.03, 128^2 3.26 -> 1.33, 200^2 4.32 -> 2.54.
+static TileGrid plan_tile(int nx, int ny, const lbm_params& p, int sms) {
+    TileGrid best = {0, 0, 0};
+    const double n = (double)nx * ny;
+    if (p.kernel == LBM_KERNEL_GENERIC || n > 1e5) return best;
+    double t = 0.95 * (p.storage == LBM_STORE_FP32 ? 2.45 + 1.5e-5 * n : 3.0 + 0.9e-5 * n);
+    for (int S = 2; S <= 6; ++S)
+        for (int h = 2; h <= 32 && h <= ny; ++h)
+            for (int w = 2; w <= 32 && w <= nx; ++w) {
+                if ((w + 4 * S - 2) * (h + 4 * S - 2) > TILE_THREADS) continue;
+                int nodes = 0;
+                for (int s = 1; s <= S; ++s) nodes += (w + 4 * (S - s) + 2) * (h + 4 * (S - s) + 2);
+                const int blocks = ((nx + w - 1) / w) * ((ny + h - 1) / h);
+                const double us = (1.78 + 2.8e-3 * nodes * ((blocks + sms - 1) / sms)) / S;
+                if (us < t) {
+                    t = us;
+                    best = TileGrid{w, h, S};
+                }
+            }
+    return best;
+}
+
+// n <= tile.S steps at once
+static lbm_status launch_tile(lbm_handle* h, int n) {
+    TileGrid G = h->tile;
+    G.S = n;
+    const dim3 grid((h->nx + G.w - 1) / G.w, (h->ny + G.h - 1) / G.h);
+    const int threads = (G.w + 4 * n - 2) * (G.h + 4 * n - 2);  // the first step's phi region
+    LBM_CUDA(h, launch_dep(tile_kernel(h->prm), grid, dim3((threads + 31) / 32 * 32), 0, h->stream, march_args(h), h->model, G,
+                           (unsigned int)h->nstep));
+    h->nstep += n;
+    h->cur ^= 1;
+    return LBM_OK;
+}
+
 // two steps at once
 static lbm_status launch_march(lbm_handle* h) {
     const int c = h->cur;
@@ -1011,12 +1099,7 @@ static lbm_status launch_march(lbm_handle* h) {
     const MarchKernel k = march_kernel(h->prm, &smem);
     MarchGrid G = h->march;
     G.par = c;
-    MarchArgs A{};
-    march_planes(h, c, (char**)A.s);
-    march_planes(h, c ^ 1, A.d);
-    A.flag = h->flag;
-    A.nx = h->nx;
-    A.ny = h->ny;
+    const MarchArgs A = march_args(h);
     h->model.seed = (unsigned int)(++h->nstep) * 0x9e3779b9u;
     const unsigned int seed2 = (unsigned int)(++h->nstep) * 0x9e3779b9u;
     const dim3 grid((h->nx + G.w - 1) / G.w, (h->ny + G.H - 1) / G.H);
@@ -1182,6 +1265,7 @@ static lbm_status create_handle(int nx, int ny, const lbm_params* p, void* ws, l
             if (st16 && !h->pm[0].on && bytes * 10.0 < (double)LBM_PREFETCH16_L2X10 * l2) h->pf_ahead = 0;
         }
     }
+    h->tile = plan_tile(nx, ny, *p, sms);
     h->march = plan_march(nx, ny, *p, sms);
     if (e == cudaSuccess && h->march.H > 0) {
         size_t smem;
@@ -1301,13 +1385,15 @@ lbm_status lbm_step(lbm_handle* h, int nsteps) {
     if (!h->inited) return fail(h, LBM_ERR_STATE, "lbm_step before lbm_init");
     LBM_CUDA(h, cudaSetDevice(h->device));
     for (int s = 0; s < nsteps;) {
-        // two steps at once, unless a check falls between them
-        const bool two = h->march.H > 0 && nsteps - s >= 2 &&
-                         (h->prm.check_every == 0 || h->prm.check_every - h->since_check >= 2);
-        lbm_status st = two ? launch_march(h) : launch_step(h, false, nullptr);
+        // several steps at once, unless a check falls between them
+        int n = nsteps - s;
+        if (h->prm.check_every > 0 && h->prm.check_every - h->since_check < n)
+            n = (int)(h->prm.check_every - h->since_check);
+        n = h->tile.S > 1 ? (n < h->tile.S ? n : h->tile.S) : h->march.H > 0 && n > 1 ? 2 : 1;
+        lbm_status st = n == 1 ? launch_step(h, false, nullptr) : h->tile.S > 1 ? launch_tile(h, n) : launch_march(h);
         if (st != LBM_OK) return st;
-        s += two ? 2 : 1;
-        if (h->prm.check_every > 0 && (h->since_check += two ? 2 : 1) >= h->prm.check_every) {
+        s += n;
+        if (h->prm.check_every > 0 && (h->since_check += n) >= h->prm.check_every) {
             st = check_flag(h);
             if (st != LBM_OK) return st;
         }
