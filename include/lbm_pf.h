@@ -258,9 +258,9 @@ lbm_status lbm_diag_fields_noalloc(const double* d_fields, size_t n, double* d_o
  * lbm_batch_step -- advance every case by nsteps time steps (the same update as
  *   lbm_step, Sec. II, bit for bit).  The cases form two classes, periodic in y
  *   and walled in y; each class has a kernel compiled for its boundary and its
- *   own stream, and one launch per step covers the tiles of all its cases.  The
- *   two classes share no data, so their launch chains run concurrently.  Steps
- *   run as replays of a CUDA graph of 32 steps per class.  The first call with
+ *   own stream, and one launch per step (per pair of steps in larger batches)
+ *   covers all its cases.  The two classes share no data, so their launch chains
+ *   run concurrently.  Steps run as replays of a CUDA graph of 32 steps per class.  The first call with
  *   nsteps >= 140 times five tile shapes (32x4, 32x8, 32x16, 64x2, 64x4 nodes)
  *   for each class on its own first 140 steps (per shape 4 warm-up steps and
  *   the faster of two windows of 12) and keeps the fastest.

@@ -98,7 +98,7 @@ __device__ __forceinline__ const T& sh(const char* p) {
 }
 
 // The pulled values of one node in a storage format: from global memory (pull;
-// s: the planes in the ring's order) or from the shared ring (pull_ring; planes
+// A.src(i): the planes in the ring's order) or from the shared ring (pull_ring; planes
 // LP bytes apart; pull_ring_phi: only what phi needs).
 template <int ST>
 struct MarchRow {  // 16-bit formats: the code words as stored
@@ -108,13 +108,14 @@ struct MarchRow {  // 16-bit formats: the code words as stored
     float f0;
     unsigned short g0;
     float2 prev;  // (phi u) of the previous step
-    template <bool WALLS>
-    __device__ __forceinline__ void pull(const char* const* s, const PullOff& o, bool lo, bool hi) {
-        prev = make_float2(ldp<float>(s[10], o.cc), ldp<float>(s[11], o.cc));
-        f0 = ldp<float>(s[0], o.cc);
-        g0 = ldp<unsigned short>(s[9], o.cc >> 1);
+    template <bool WALLS, class ARGS>
+    __device__ __forceinline__ void pull(const ARGS& A, const PullOff& o, bool lo, bool hi) {
+        prev = make_float2(ldp<float>(A.src(10), o.cc), ldp<float>(A.src(11), o.cc));
+        f0 = ldp<float>(A.src(0), o.cc);
+        g0 = ldp<unsigned short>(A.src(9), o.cc >> 1);
         w[0] = 0u;
-        pull_dirs<WALLS, false>([&](int i, unsigned int off) { return ldp<unsigned int>(s[i], off); }, o, lo, hi, w);
+        pull_dirs<WALLS, false>([&](int i, unsigned int off) { return ldp<unsigned int>(A.src(i), off); }, o, lo, hi,
+                                w);
     }
     template <bool WALLS, int LP>
     __device__ __forceinline__ void pull_ring_phi(const char* ring, const PullOff& o, bool lo, bool hi) {
@@ -153,18 +154,19 @@ struct MarchRow {  // 16-bit formats: the code words as stored
         sh<float>(at + 10 * LP) = pu.x;
         sh<float>(at + 11 * LP) = pu.y;
     }
-    __device__ static __forceinline__ void put(char* const* d, unsigned int off, const float h[9], const float k[9],
+    template <class ARGS>
+    __device__ static __forceinline__ void put(const ARGS& A, unsigned int off, const float h[9], const float k[9],
                                                float phi, float2 pu, unsigned int seed) {
         unsigned int w[9];
         float r0;
         unsigned short q0;
         P::template encode<MARCH_PK>(h, k, phi, off >> 2, seed, w, r0, q0);
 #pragma unroll
-        for (int i = 1; i < 9; ++i) stp(d[i], off, w[i]);
-        stp(d[0], off, r0);
-        stp(d[9], off >> 1, q0);
-        stp(d[10], off, pu.x);
-        stp(d[11], off, pu.y);
+        for (int i = 1; i < 9; ++i) stp(A.dst(i), off, w[i]);
+        stp(A.dst(0), off, r0);
+        stp(A.dst(9), off >> 1, q0);
+        stp(A.dst(10), off, pu.x);
+        stp(A.dst(11), off, pu.y);
     }
 };
 template <>
@@ -172,11 +174,11 @@ struct MarchRow<ST_FP32> {
     static constexpr int RING_PLANES = 20;  // f, g, (phi u)
     float f[9], g[9];
     float2 prev;
-    template <bool WALLS>
-    __device__ __forceinline__ void pull(const char* const* s, const PullOff& o, bool lo, bool hi) {
-        prev = make_float2(ldp<float>(s[18], o.cc), ldp<float>(s[19], o.cc));
-        pull_dirs<WALLS, true>([&](int i, unsigned int off) { return ldp<float>(s[i], off); }, o, lo, hi, f);
-        pull_dirs<WALLS, true>([&](int i, unsigned int off) { return ldp<float>(s[9 + i], off); }, o, lo, hi, g);
+    template <bool WALLS, class ARGS>
+    __device__ __forceinline__ void pull(const ARGS& A, const PullOff& o, bool lo, bool hi) {
+        prev = make_float2(ldp<float>(A.src(18), o.cc), ldp<float>(A.src(19), o.cc));
+        pull_dirs<WALLS, true>([&](int i, unsigned int off) { return ldp<float>(A.src(i), off); }, o, lo, hi, f);
+        pull_dirs<WALLS, true>([&](int i, unsigned int off) { return ldp<float>(A.src(9 + i), off); }, o, lo, hi, g);
     }
     template <bool WALLS, int LP>
     __device__ __forceinline__ void pull_ring_phi(const char* ring, const PullOff& o, bool lo, bool hi) {
@@ -208,30 +210,33 @@ struct MarchRow<ST_FP32> {
         sh<float>(at + 18 * LP) = pu.x;
         sh<float>(at + 19 * LP) = pu.y;
     }
-    __device__ static __forceinline__ void put(char* const* d, unsigned int off, const float h[9], const float k[9],
+    template <class ARGS>
+    __device__ static __forceinline__ void put(const ARGS& A, unsigned int off, const float h[9], const float k[9],
                                                float phi, float2 pu, unsigned int) {
-        stp(d[0], off, sub(phi, sum8<MARCH_PK>(h)));
-        stp(d[9], off, k[0]);
+        stp(A.dst(0), off, sub(phi, sum8<MARCH_PK>(h)));
+        stp(A.dst(9), off, k[0]);
 #pragma unroll
         for (int i = 1; i < 9; ++i) {
-            stp(d[i], off, h[i]);
-            stp(d[9 + i], off, k[i]);
+            stp(A.dst(i), off, h[i]);
+            stp(A.dst(9 + i), off, k[i]);
         }
-        stp(d[18], off, pu.x);
-        stp(d[19], off, pu.y);
+        stp(A.dst(18), off, pu.x);
+        stp(A.dst(19), off, pu.y);
     }
 };
 
 constexpr int MARCH_HALO = 3;  // columns and rows computed beyond a block's own on each side
-constexpr int MARCH_PAD = 1;   // floats before and after each row of the shared arrays
+constexpr int MARCH_PAD = 16;  // bytes before and after the shared rows: the outermost threads read one past them
 
 template <int TW, int ST>
 struct MarchSmem {
-    static constexpr int LINE = 4 * (TW + 2 * MARCH_PAD);              // bytes of one row of one plane
-    static constexpr int SLOT = LINE * MarchRow<ST>::RING_PLANES;      // one ring row
-    static constexpr int PHI = 0;                                      // the newest phi row of step 1, of step 2
-    static constexpr int RING = 6 * LINE;
-    static constexpr int BYTES = RING + 5 * SLOT;
+    static constexpr int LINE = 4 * TW;                            // bytes of one row of one plane
+    static constexpr int SLOT = LINE * MarchRow<ST>::RING_PLANES;  // one ring row
+    static constexpr int PHI = MARCH_PAD;                          // phi of step 1, 3 rows, then of step 2
+    static constexpr int RING = PHI + 6 * LINE;
+    // FP32: 54.3 KB, so that three blocks stay within a 164 KB share of the SM's
+    // 256 KB and leave the L1 cache 92 KB
+    static constexpr int BYTES = RING + 5 * SLOT + MARCH_PAD;
 };
 
 // The planes read and written, in the ring's order (the addresses come from the
@@ -241,14 +246,32 @@ struct MarchArgs {
     char* d[20];
     unsigned int* flag;
     int nx, ny;
+    __device__ __forceinline__ const char* src(int i) const { return s[i]; }
+    __device__ __forceinline__ char* dst(int i) const { return d[i]; }
+};
+// The same of one case of a batch, from its buffers' bases.
+template <int ST>
+struct MarchCase {
+    const char *fs, *gs, *pus;
+    char *fd, *gd, *pud;
+    size_t plane;  // bytes of a plane of 4-byte entries
+    unsigned int* flag;
+    int nx, ny;
+    static constexpr int G = ST == ST_FP32 ? 9 : 1;  // planes of the g buffer
+    __device__ __forceinline__ const char* src(int i) const {
+        return i < 9 ? fs + i * plane : i < 9 + G ? gs + (i - 9) * plane : pus + (i - 9 - G) * plane;
+    }
+    __device__ __forceinline__ char* dst(int i) const {
+        return i < 9 ? fd + i * plane : i < 9 + G ? gd + (i - 9) * plane : pud + (i - 9 - G) * plane;
+    }
 };
 
 // One block's strip of columns [x0, x0 + wlen) and chunk of rows [y0, y1),
 // marched in direction dir.  m.seed / seed2: the
 // dithers' seeds of the two steps.
 // STEP: which of the two steps the calling threads take.
-template <int STEP, int TW, int WALLS, int ST, bool CHK>
-__device__ __forceinline__ void march_block(char* smem, const MarchArgs& A, const Model& m, int x0, int wlen,
+template <int STEP, int TW, int WALLS, int ST, bool CHK, class ARGS>
+__device__ __forceinline__ void march_block(char* smem, const ARGS& A, const Model& m, int x0, int wlen,
                                             int y0, int y1, int dir, unsigned int seed2) {
     using Row = MarchRow<ST>;
     using S = MarchSmem<TW, ST>;
@@ -268,7 +291,7 @@ __device__ __forceinline__ void march_block(char* smem, const MarchArgs& A, cons
         return t >= 3 - k && t <= rows + 2 + k && (!W || (unsigned)y < (unsigned)ny);
     };
 
-    char* const sx = smem + 4 * (MARCH_PAD + tx);  // this thread's column in row 0 of plane 0
+    char* const sx = smem + 4 * tx;  // this thread's column of every row
 #if LBM_DEBUG_CHECKS
     for (int k = threadIdx.x; k < S::BYTES / 4; k += 2 * TW)
         reinterpret_cast<float*>(smem)[k] = __int_as_float(0x7fc00000);
@@ -300,7 +323,7 @@ __device__ __forceinline__ void march_block(char* smem, const MarchArgs& A, cons
         constexpr bool WB = W && !decltype(fast)::value;
         const int y = wrap(yl);
         if (row_bad(y)) return;
-        R.template pull<WB>(A.s, row_off(fast, y), WB && y == 0, WB && !open_top && y == ny - 1);
+        R.template pull<WB>(A, row_off(fast, y), WB && y == 0, WB && !open_top && y == ny - 1);
     };
     // ring offsets of rows y-1, y, y+1 (slots given for the logical rows before
     // and after, which are y-1 and y+1 or the reverse)
@@ -360,7 +383,7 @@ __device__ __forceinline__ void march_block(char* smem, const MarchArgs& A, cons
         const Stencil st = stencil_rows(fast, b, c, a, y);
         const Macro M = macro_from<MARCH_PK>(m, Pop<ST>::template gmom<MARCH_PK>(g), phi, st.gx, st.gy, st.lap);
         if constexpr (CHK)
-            if (own && !isfinite(add(add(phi, M.ux), add(M.uy, M.p)))) report_nonfinite(A.flag);
+            if (own && m.check_nonfinite && !isfinite(add(add(phi, M.ux), add(M.uy, M.p)))) report_nonfinite(A.flag);
         return collide_st<ST, MARCH_PK>(m, f, g, phi, st, M, R.prev);
     };
     std::false_type edge;
@@ -416,7 +439,7 @@ __device__ __forceinline__ void march_block(char* smem, const MarchArgs& A, cons
                 float f[9], g[9], phi;
                 const float2 pu = collide_row(fast, R, row3(phis + a2), row3(phis + a1), row3(phis + a0), yc, out, f,
                                               g, phi);
-                if (out) Row::put(A.d, pitch * yc + xc, f, g, phi, pu, seed2);
+                if (out) Row::put(A, pitch * yc + xc, f, g, phi, pu, seed2);
             }
             sync_block();
             rotate();

@@ -135,9 +135,8 @@ __device__ __forceinline__ bool nbr_in_range(const Nbr& q, int nx, int ny) {
 template <int TX, int TY, bool FIELDS, int WALLS, int ST, bool CHK>
 __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __restrict__ fs,
                                           const float* __restrict__ gs, float* __restrict__ fd,
-                                          float* __restrict__ gd, const float* __restrict__ pus,
-                                          float* __restrict__ pud, unsigned int* __restrict__ flag,
-                                          double* __restrict__ out,
+                                          float* __restrict__ gd, float* __restrict__ phiu,
+                                          unsigned int* __restrict__ flag, double* __restrict__ out,
                                           int nx, int ny, Model m, int x0, int y0) {
     if (WALLS == 0) m.walls = 0;  // WALLS == 1 keeps the kind of top (wall or open)
     const int wfold = WALLS >= 0 ? WALLS : m.walls;  // y folding: wrap (0) or clamp
@@ -171,7 +170,7 @@ __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __
         }
 #endif
 #if LBM_EARLY_PHIU
-        if (!FIELDS) prev = make_float2(pus[q.r0 + x], pus[N32 + q.r0 + x]);
+        if (!FIELDS) prev = make_float2(phiu[q.r0 + x], phiu[N32 + q.r0 + x]);
 #endif
         pull18<ST, WALLS>(fs, gs, N32, q, f, g);
         sphi[ty + 1][tx + 1] = Pop<ST>::phi_of(f);
@@ -217,11 +216,11 @@ __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __
     if constexpr (CHK) bad = m.check_nonfinite && !isfinite(add(add(phi, M.ux), add(M.uy, M.p)));
 
 #if !LBM_EARLY_PHIU
-    const float2 prev = make_float2(pus[n32], pus[N32 + n32]);
+    const float2 prev = make_float2(phiu[n32], phiu[N32 + n32]);
 #endif
     const float2 now = collide_st<ST>(m, f, g, phi, st, M, prev);
-    pud[n32] = now.x;
-    pud[N32 + n32] = now.y;
+    phiu[n32] = now.x;
+    phiu[N32 + n32] = now.y;
     Pop<ST>::stfg(fd, gd, N32, n32, f, g, phi);
     if constexpr (CHK)
         if (bad) report_nonfinite(flag);
@@ -239,9 +238,9 @@ __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __
 template <int TX, int TY, int NPT, int WALLS, int ST, bool CHK>
 __device__ __forceinline__ void step_tile16(float (*sphi)[TX + 2], const void* __restrict__ fs,
                                             const void* __restrict__ gs, void* __restrict__ fd,
-                                            void* __restrict__ gd, const float* __restrict__ pus,
-                                            float* __restrict__ pud, unsigned int* __restrict__ flag,
-                                            int nx, int ny, Model m, int x0, int y0) {
+                                            void* __restrict__ gd, float* __restrict__ phiu,
+                                            unsigned int* __restrict__ flag, int nx, int ny, Model m,
+                                            int x0, int y0) {
     constexpr bool BR = (WALLS < 0) || LBM_WALL_BRANCH;
     constexpr int TH = TY * NPT;
     if (WALLS == 0) m.walls = 0;  // WALLS == 1 keeps the kind of top (wall or open)
@@ -275,7 +274,7 @@ __device__ __forceinline__ void step_tile16(float (*sphi)[TX + 2], const void* _
             }
 #endif
             n[j] = q.r0 + q.x;
-            prev[j] = make_float2(pus[n[j]], pus[N + n[j]]);
+            prev[j] = make_float2(phiu[n[j]], phiu[N + n[j]]);
             pull_words16<ST, BR, true>(fs, gs, N, q, w[j], f0[j], g0[j]);
             float h[9];
             codes_f<ST>(w[j], f0[j], h);
@@ -314,8 +313,8 @@ __device__ __forceinline__ void step_tile16(float (*sphi)[TX + 2], const void* _
         bool bad = false;
         if constexpr (CHK) bad = m.check_nonfinite && !isfinite(add(add(phi, M.ux), add(M.uy, M.p)));
         const float2 now = collide_code<Pop<ST>>(m, h, k, phi, st, M, prev[j]);
-        pud[n[j]] = now.x;
-        pud[N + n[j]] = now.y;
+        phiu[n[j]] = now.x;
+        phiu[N + n[j]] = now.y;
         Pop<ST>::stfg(fd, gd, N, n[j], h, k, phi, m.seed);
         if constexpr (CHK)
             if (bad) report_nonfinite(flag);
@@ -422,10 +421,7 @@ __device__ __forceinline__ void prefetch_tile(const void* fs, const void* gs, co
 #ifndef LBM_MARCH_THREADS16
 #define LBM_MARCH_THREADS16 768
 #endif
-#ifndef LBM_MARCH_MIN_EFF
-#define LBM_MARCH_MIN_EFF 0.40
-#endif
-constexpr double MARCH_MIN_EFF = LBM_MARCH_MIN_EFF;
+constexpr double MARCH_BATCH_MIN_SHARE = 0.40, MARCH_BATCH_MIN_SHARE16 = 0.62;  // see plan_march_batch
 // Resident blocks per SM each step kernel is compiled for (its register
 // budget), measured per instantiation with 32 x 4 tiles at 2048^2 (2400 x 600
 // for walls), MLUPS at 8 / 9 / 10 blocks:
@@ -454,8 +450,8 @@ __host__ __device__ constexpr int step_npt() {
 template <int TX, int TY, bool FIELDS, int WALLS, int ST, bool CHK = false>
 __global__ void __launch_bounds__(TX* TY, (step_minb<FIELDS, WALLS, ST, TX * TY>()))
     k_step(const float* __restrict__ fs, const float* __restrict__ gs, float* __restrict__ fd,
-           float* __restrict__ gd, const float* __restrict__ pus, float* __restrict__ pud,
-           unsigned int* __restrict__ flag, double* __restrict__ out, int nx, int ny, Model m, int pf_ahead, int rev,
+           float* __restrict__ gd, float* __restrict__ phiu, unsigned int* __restrict__ flag,
+           double* __restrict__ out, int nx, int ny, Model m, int pf_ahead, int rev,
            const __grid_constant__ PfMaps pm) {
     constexpr int NPT = step_npt<FIELDS, ST>();
     __shared__ float sphi[TY * NPT + 2][TX + 2];
@@ -478,16 +474,16 @@ __global__ void __launch_bounds__(TX* TY, (step_minb<FIELDS, WALLS, ST, TX * TY>
                 if (pm.on)
                     prefetch_tile_maps<TY * NPT, ST>(pm, px * TX, py);
                 else
-                    prefetch_tile<TX, TY * NPT, TX * TY, ST>(fs, gs, pus, nx, ny,
+                    prefetch_tile<TX, TY * NPT, TX * TY, ST>(fs, gs, phiu, nx, ny,
                                                              WALLS >= 0 ? WALLS : m.walls, px, py);
             }
         }
     }
     if constexpr (NPT > 1 || (!FIELDS && ST != ST_FP32))
-        step_tile16<TX, TY, NPT, WALLS, ST, CHK>(sphi, fs, gs, fd, gd, pus, pud, flag, nx, ny, m,
+        step_tile16<TX, TY, NPT, WALLS, ST, CHK>(sphi, fs, gs, fd, gd, phiu, flag, nx, ny, m,
                                                  bx * TX, by * TY * NPT);
     else
-        step_tile<TX, TY, FIELDS, WALLS, ST, CHK>(sphi, fs, gs, fd, gd, pus, pud, flag, out, nx, ny, m,
+        step_tile<TX, TY, FIELDS, WALLS, ST, CHK>(sphi, fs, gs, fd, gd, phiu, flag, out, nx, ny, m,
                                                   bx * TX, by * TY);
 }
 
@@ -760,11 +756,12 @@ struct lbm_handle {
     cudaStream_t stream = nullptr;
     float* f[2] = {nullptr, nullptr};
     float* g[2] = {nullptr, nullptr};
-    // (phi u) of the previous step, going with the population buffer of the
-    // same index; phiu[1] lives in the last 2 N floats of the staging buffer,
-    // where a checkpoint keeps it (no read-back writes there before reading it)
+    // (phi u) of the previous step, in phiu[pcur]: a one-step launch updates it in
+    // place, a launch of several steps writes the other buffer.  phiu[1] lives in
+    // the last 2 N floats of the staging buffer, where a checkpoint keeps it (no
+    // read-back writes there before reading it).
     float* phiu[2] = {nullptr, nullptr};
-    int cur = 0;
+    int cur = 0, pcur = 0;
     void* staging = nullptr;   // host I/O staging: max(5 N doubles, 20 N floats)
     double* red_part = nullptr;  // RED_BLOCKS x 4 partials
     double* red_res = nullptr;   // 4 results
@@ -775,6 +772,7 @@ struct lbm_handle {
     bool owns_memory = true;  // false: the device buffers live in a caller's workspace
     unsigned long long nstep = 0;  // steps since lbm_init: seeds the stochastic rounding
     PfMaps pm[2] = {};             // prefetch tensor maps of the step reading buffer 0 / 1
+    CUtensorMap pm_phiu1 = {};     // the (phi u) map of phiu[1] (pm's are of phiu[0])
     TileGrid tile = {0, 0, 0};     // tiles of the several-step kernel (S = 0: not used)
     MarchGrid march = {0, 0, 0};   // strips and chunks of the two-step kernel (H = 0: not used)
     char err[512] = {0};
@@ -939,7 +937,7 @@ static lbm_status launch_step(lbm_handle* h, bool fields, double* out) {
     const int th = st16 ? STEP_TY * LBM_NPT16 : STEP_TY;
     dim3 block(tw, STEP_TY);
     dim3 grid((h->nx + tw - 1) / tw, (h->ny + th - 1) / th);
-    using K = void (*)(const float*, const float*, float*, float*, const float*, float*, unsigned int*, double*,
+    using K = void (*)(const float*, const float*, float*, float*, float*, unsigned int*, double*,
                        int, int, Model, int, int, PfMaps);
     K k;
     // the steps of a handle that asked for non-finite checks test every node;
@@ -962,16 +960,17 @@ static lbm_status launch_step(lbm_handle* h, bool fields, double* out) {
     }
 #undef LBM_STEP_KERNEL
     if (fields)
-        k<<<grid, block, 0, h->stream>>>(h->f[c], h->g[c], nullptr, nullptr, h->phiu[c], nullptr, h->flag,
-                                         out, h->nx, h->ny, h->model, 0, 0, PfMaps{});
+        k<<<grid, block, 0, h->stream>>>(h->f[c], h->g[c], nullptr, nullptr, h->phiu[h->pcur], h->flag, out,
+                                         h->nx, h->ny, h->model, 0, 0, PfMaps{});
     else {
+        PfMaps pm = h->pm[c];
+        if (h->pcur) pm.phiu = h->pm_phiu1;
         // a distinct seed per step (the golden-ratio multiple of the step count)
         h->model.seed = (unsigned int)(++h->nstep) * 0x9e3779b9u;
         LBM_CUDA(h, launch_dep(k, grid, block, 0, h->stream, (const float*)h->f[c],
-                               (const float*)h->g[c], h->f[c ^ 1], h->g[c ^ 1],
-                               (const float*)h->phiu[c], h->phiu[c ^ 1], h->flag,
+                               (const float*)h->g[c], h->f[c ^ 1], h->g[c ^ 1], h->phiu[h->pcur], h->flag,
                                (double*)nullptr, h->nx, h->ny, h->model, h->pf_ahead,
-                               LBM_ALTERNATE_ORDER ? c : 0, h->pm[c]));
+                               LBM_ALTERNATE_ORDER ? c : 0, pm));
     }
     LBM_CUDA(h, cudaGetLastError());
     if (!fields) h->cur ^= 1;
@@ -997,8 +996,14 @@ static MarchKernel march_kernel(const lbm_params& p, size_t* smem) {
 }
 
 // Strips and chunks of a handle's two-step launches: one resident wave of
-// blocks.  A block computes TW columns for w of its own and about H + 7 rows'
-// time for H, so the march pays where w / TW * H / (H + 7) is high enough.
+// blocks.  A block computes TW columns for w of its own and takes about H + 7
+// rows' time for H, so the march pays where eff = w / TW * H / (H + 7) is high
+// enough.  One-step time / march time at eff, nx a multiple of 8: FP32 640 x 400
+// 0.39 0.92, 560^2 0.44 1.02, 704^2 0.54 1.09, 1000 x 600 0.55 1.26, 960^2 0.66
+// 1.46; FP16 800 x 500 0.48 0.97, 768^2 0.54 0.95, 1000 x 600 0.55 1.03, 960^2 0.66
+// 1.07.  Other nx, whose rows start inside a 32-byte sector, slow the one-step
+// kernels down: FP32 501^2 0.36 1.13, 901 x 300 0.41 1.18; FP16 901 x 300 0.41 0.99,
+// 601^2 0.47 1.19.
 static MarchGrid plan_march(int nx, int ny, const lbm_params& p, int sms) {
     MarchGrid g = {0, 0, 0};
     if (p.kernel == LBM_KERNEL_GENERIC || nx < 64 || ny < 16) return g;
@@ -1009,23 +1014,22 @@ static MarchGrid plan_march(int nx, int ny, const lbm_params& p, int sms) {
     const int chunks = sms * per_sm / strips > 1 ? sms * per_sm / strips : 1;
     g.H = (ny + chunks - 1) / chunks;
     const double eff = (double)g.w / MARCH_TW * g.H / (g.H + 7);
-    if (eff < MARCH_MIN_EFF) g.H = 0;
+    const bool fp32 = p.storage == LBM_STORE_FP32;
+    if (eff < (nx % 8 == 0 ? (fp32 ? 0.43 : 0.55) : (fp32 ? 0.36 : 0.42))) g.H = 0;
     return g;
 }
 
-// the planes of buffer c in the march's order (MarchArgs)
-static void march_planes(const lbm_handle* h, int c, char* p[20]) {
-    const bool st16 = h->prm.storage != LBM_STORE_FP32;
-    const int nf = 9, ng = st16 ? 1 : 9;
+// the planes of population buffer c and (phi u) buffer pc in the march's order
+static void march_planes(const lbm_handle* h, int c, int pc, char* p[20]) {
+    const int nf = 9, ng = h->prm.storage == LBM_STORE_FP32 ? 9 : 1;
     for (int i = 0; i < nf; ++i) p[i] = (char*)(h->f[c] + i * h->N);
     for (int i = 0; i < ng; ++i) p[nf + i] = (char*)(h->g[c] + i * h->N);
-    for (int i = 0; i < 2; ++i) p[nf + ng + i] = (char*)(h->phiu[c] + i * h->N);
+    for (int i = 0; i < 2; ++i) p[nf + ng + i] = (char*)(h->phiu[pc] + i * h->N);
 }
-
 static MarchArgs march_args(const lbm_handle* h) {
     MarchArgs A{};
-    march_planes(h, h->cur, (char**)A.s);
-    march_planes(h, h->cur ^ 1, A.d);
+    march_planes(h, h->cur, h->pcur, (char**)A.s);
+    march_planes(h, h->cur ^ 1, h->pcur ^ 1, A.d);
     A.flag = h->flag;
     A.nx = h->nx;
     A.ny = h->ny;
@@ -1089,6 +1093,7 @@ static lbm_status launch_tile(lbm_handle* h, int n) {
                            (unsigned int)h->nstep));
     h->nstep += n;
     h->cur ^= 1;
+    h->pcur ^= 1;
     return LBM_OK;
 }
 
@@ -1105,6 +1110,7 @@ static lbm_status launch_march(lbm_handle* h) {
     const dim3 grid((h->nx + G.w - 1) / G.w, (h->ny + G.H - 1) / G.H);
     LBM_CUDA(h, launch_dep(k, grid, dim3(2 * MARCH_TW), smem, h->stream, A, h->model, G, seed2));
     h->cur ^= 1;
+    h->pcur ^= 1;
     return LBM_OK;
 }
 
@@ -1171,15 +1177,15 @@ static bool encode_prefetch_map(CUtensorMap* m, CUtensorMapDataType t, int es, v
 }
 
 // The four 16-bit prefetch maps of buffer c of handle h (word planes, f_0,
-// g_0, (phi u)), box bx x by
-static bool encode_maps16(const lbm_handle* h, int c, CUtensorMap m[4], int bx, int by) {
+// g_0, (phi u) in its buffer pc), box bx x by
+static bool encode_maps16(const lbm_handle* h, int c, int pc, CUtensorMap m[4], int bx, int by) {
     const int nx = h->nx, ny = h->ny;
     const size_t N = h->N;
     return encode_prefetch_map(&m[0], CU_TENSOR_MAP_DATA_TYPE_UINT32, 4,
                                static_cast<char*>((void*)h->f[c]) + 4 * N, 8, nx, ny, bx, by) &&
            encode_prefetch_map(&m[1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->f[c], 1, nx, ny, bx, by) &&
            encode_prefetch_map(&m[2], CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, h->g[c], 1, nx, ny, bx, by) &&
-           encode_prefetch_map(&m[3], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu[c], 2, nx, ny, bx, by);
+           encode_prefetch_map(&m[3], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu[pc], 2, nx, ny, bx, by);
 }
 
 static void encode_pf_maps(lbm_handle* h) {
@@ -1196,7 +1202,7 @@ static void encode_pf_maps(lbm_handle* h) {
         bool ok;
         if (st16) {
             CUtensorMap m[4];
-            ok = encode_maps16(h, c, m, tx, th + 2);
+            ok = encode_maps16(h, c, 0, m, tx, th + 2);
             if (ok) {
                 pm.pop[0] = m[0];
                 pm.pop[1] = m[1];
@@ -1208,9 +1214,11 @@ static void encode_pf_maps(lbm_handle* h) {
                                      tx, th + 2) &&
                  encode_prefetch_map(&pm.pop[1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->g[c], 9, nx, ny,
                                      tx, th + 2) &&
-                 encode_prefetch_map(&pm.phiu, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu[c], 2, nx, ny,
+                 encode_prefetch_map(&pm.phiu, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu[0], 2, nx, ny,
                                      tx, th + 2);
         }
+        ok = ok && encode_prefetch_map(&h->pm_phiu1, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, h->phiu[1], 2, nx, ny, tx,
+                                       th + 2);
         if (!ok) {
             h->pm[0].on = h->pm[1].on = 0;
             return;
@@ -1364,7 +1372,7 @@ lbm_status lbm_init(lbm_handle* h, const double* phi0, const double* ux0, const 
         else
             LBM_CUDA(h, cudaMemsetAsync(in + k * h->N, 0, bytes, h->stream));
     }
-    h->cur = 0;
+    h->cur = h->pcur = 0;
     auto kinit = h->prm.storage == LBM_STORE_FP16_SHIFTED ? k_init<ST_FP16>
                  : is_bf16(h->prm.storage)                ? k_init<ST_BF16>
                                                           : k_init<ST_FP32>;
@@ -1429,7 +1437,7 @@ lbm_status lbm_get_state(lbm_handle* h, void* host_buf, size_t bytes) {
     auto kout = h->prm.storage == LBM_STORE_FP16_SHIFTED ? k_state_out<ST_FP16>
                 : is_bf16(h->prm.storage)                ? k_state_out<ST_BF16>
                                                           : k_state_out<ST_FP32>;
-    kout<<<grid1d(h->N), 256, 0, h->stream>>>(h->f[h->cur], h->g[h->cur], h->phiu[h->cur], st,
+    kout<<<grid1d(h->N), 256, 0, h->stream>>>(h->f[h->cur], h->g[h->cur], h->phiu[h->pcur], st,
                                                       h->nx, h->ny, h->model.walls);
     LBM_CUDA(h, cudaGetLastError());
     LBM_CUDA(h, cudaMemcpyAsync(host_buf, st, bytes, cudaMemcpyDeviceToHost, h->stream));
@@ -1445,7 +1453,7 @@ lbm_status lbm_set_state(lbm_handle* h, const void* host_buf, size_t bytes) {
     LBM_CUDA(h, cudaSetDevice(h->device));
     float* st = (float*)h->staging;
     LBM_CUDA(h, cudaMemcpyAsync(st, host_buf, bytes, cudaMemcpyHostToDevice, h->stream));
-    h->cur = 0;
+    h->cur = h->pcur = 0;
     auto kin = h->prm.storage == LBM_STORE_FP16_SHIFTED ? k_state_in<ST_FP16>
                : is_bf16(h->prm.storage)                ? k_state_in<ST_BF16>
                                                          : k_state_in<ST_FP32>;
@@ -1659,7 +1667,7 @@ struct CaseDesc {
     float* phiu[2];
     unsigned int* flag;
     int nx, ny;
-    int cur;   // buffer holding the current state when the batch parity is 0
+    int cur;   // buffers holding the current state when the batch parities are 0 (bits as parity's)
     int map0;  // first of the case's 8 prefetch maps in BatchTable::maps (4 per buffer)
     Model m;
 };
@@ -1699,7 +1707,8 @@ static_assert(sizeof(BatchTable) <= 32000, "kernel parameters are limited to 32 
 #define LBM_BATCH_THREADS16 1024
 #endif
 
-// One time step of every case of one boundary class (WALLS = 0: periodic in
+// One time step of every case of one boundary class (parity: bit 0 of the
+// population buffers, bit 1 of the (phi u) buffers; WALLS = 0: periodic in
 // y, 1: walls in y): block t runs tile t of the class's tile list, whose
 // entry holds (case, tile row << 16 | tile column).
 template <int TX, int TY, int ST, int WALLS, bool CHK>
@@ -1739,7 +1748,7 @@ __global__ void __launch_bounds__(TX* TY, (ST == ST_FP32 ? LBM_BATCH_THREADS : L
                     tma_prefetch_3d(mp, x, y, 0);
             }
         } else {
-            prefetch_tile<TX, TH, TX * TY, ST>(pc.f[pcur], pc.g[pcur], pc.phiu[pcur], pc.nx, pc.ny, WALLS,
+            prefetch_tile<TX, TH, TX * TY, ST>(pc.f[pcur], pc.g[pcur], pc.phiu[((pc.cur >> 1) + (parity >> 1)) & 1], pc.nx, pc.ny, WALLS,
                                                pe.y & 0xffff, pe.y >> 16);
         }
     }
@@ -1755,15 +1764,42 @@ __global__ void __launch_bounds__(TX* TY, (ST == ST_FP32 ? LBM_BATCH_THREADS : L
 #endif
     const CaseDesc& cd = T.c[e.x];
     const int c = (cd.cur + parity) & 1;
+    float* const pu = cd.phiu[((cd.cur >> 1) + (parity >> 1)) & 1];
     if constexpr (ST == ST_FP32) {
-        step_tile<TX, TY, false, WALLS, ST, CHK>(sphi, cd.f[c], cd.g[c], cd.f[c ^ 1], cd.g[c ^ 1],
-                                                 cd.phiu[c], cd.phiu[c ^ 1], cd.flag, nullptr, cd.nx, cd.ny, cd.m, (e.y & 0xffff) * TX,
+        step_tile<TX, TY, false, WALLS, ST, CHK>(sphi, cd.f[c], cd.g[c], cd.f[c ^ 1], cd.g[c ^ 1], pu,
+                                                 cd.flag, nullptr, cd.nx, cd.ny, cd.m, (e.y & 0xffff) * TX,
                                             (e.y >> 16) * TY);
     } else {
         step_tile16<TX, TY, LBM_NPT16_BATCH, WALLS, ST, CHK>(
-            sphi, cd.f[c], cd.g[c], cd.f[c ^ 1], cd.g[c ^ 1], cd.phiu[c], cd.phiu[c ^ 1], cd.flag, cd.nx, cd.ny, cd.m,
+            sphi, cd.f[c], cd.g[c], cd.f[c ^ 1], cd.g[c ^ 1], pu, cd.flag, cd.nx, cd.ny, cd.m,
             (e.y & 0xffff) * TX, (e.y >> 16) * TY * LBM_NPT16_BATCH);
     }
+}
+
+// Two time steps of every case of one boundary class: block t takes entry t of
+// the class's list, (case, first column, first row, columns << 16 | rows), as
+// k_march takes a strip's chunk.
+template <int ST, int WALLS, bool CHK>
+__global__ void __launch_bounds__(2 * MARCH_TW, march_minb<ST>())
+    k_march_batch(const __grid_constant__ BatchTable T, const int4* __restrict__ list, int parity) {
+    extern __shared__ __align__(16) char march_smem[];
+    griddep_wait();
+    griddep_launch();
+    const int4 e = __ldg(list + blockIdx.x);
+    // (broadcast, so that the compiler sees warp-uniform values)
+    const int cs = __shfl_sync(0xffffffffu, e.x, 0), x0 = __shfl_sync(0xffffffffu, e.y, 0);
+    const int y0 = __shfl_sync(0xffffffffu, e.z & 0x7fffffff, 0), wh = __shfl_sync(0xffffffffu, e.w, 0);
+    const int odd = __shfl_sync(0xffffffffu, (int)((unsigned)e.z >> 31), 0);
+    const CaseDesc& cd = T.c[cs];
+    const int c = (cd.cur + parity) & 1;
+    const int pc = ((cd.cur >> 1) + (parity >> 1)) & 1;
+    const MarchCase<ST> A{(const char*)cd.f[c], (const char*)cd.g[c], (const char*)cd.phiu[pc], (char*)cd.f[c ^ 1],
+                          (char*)cd.g[c ^ 1], (char*)cd.phiu[pc ^ 1], (size_t)4 * cd.nx * cd.ny, cd.flag, cd.nx, cd.ny};
+    const int wlen = wh >> 16, y1 = y0 + (wh & 0xffff), dir = (odd + c) & 1 ? -1 : 1;
+    if (__shfl_sync(0xffffffffu, (int)threadIdx.x, 0) < MARCH_TW)
+        march_block<1, MARCH_TW, WALLS, ST, CHK>(march_smem, A, cd.m, x0, wlen, y0, y1, dir, 0u);
+    else
+        march_block<2, MARCH_TW, WALLS, ST, CHK>(march_smem, A, cd.m, x0, wlen, y0, y1, dir, 0u);
 }
 
 // boundary classes: each has its own specialised kernel, stream and tile shape
@@ -1806,6 +1842,19 @@ BatchKernel batch_kernel_for(int storage, int cls, int cand, bool chk) {
     return batch_kernel_st<ST_FP32>(cls, cand, chk);
 }
 
+using MarchBatchKernel = void (*)(BatchTable, const int4*, int);
+template <int ST>
+MarchBatchKernel march_batch_st(int cls, bool chk) {
+    if (chk) return cls ? k_march_batch<ST, 1, true> : k_march_batch<ST, 0, true>;
+    return cls ? k_march_batch<ST, 1, false> : k_march_batch<ST, 0, false>;
+}
+MarchBatchKernel march_batch_kernel(int storage, int cls, bool chk, size_t* smem) {
+    *smem = storage == LBM_STORE_FP32 ? MarchSmem<MARCH_TW, ST_FP32>::BYTES : MarchSmem<MARCH_TW, ST_FP16>::BYTES;
+    if (storage == LBM_STORE_FP16_SHIFTED) return march_batch_st<ST_FP16>(cls, chk);
+    if (storage == LBM_STORE_BF16_SHIFTED) return march_batch_st<ST_BF16>(cls, chk);
+    return march_batch_st<ST_FP32>(cls, chk);
+}
+
 // Copy the non-finite flags of one class's cases to out[slot[j]] and clear
 // them (one thread per case).
 __global__ void k_batch_flags(const __grid_constant__ BatchTable T, const int* __restrict__ slot,
@@ -1839,6 +1888,8 @@ struct lbm_batch {
     int cand[BATCH_NCLASS] = {1, 1};  // tile shape in use per class (index into BATCH_TX/TY)
     int pf_ahead = 0;                 // L2 prefetch distance in tiles (0: off)
     CUtensorMap* d_maps = nullptr;    // the 16-bit prefetch maps, 8 per case (nullptr: none)
+    int4* d_march[BATCH_NCLASS] = {};  // the two-step kernel's block lists, and their lengths
+    int march[BATCH_NCLASS] = {0, 0};  // (0 in both: not used)
     bool tuned = false;
     double tuned_us[BATCH_NCLASS][BATCH_NCAND] = {};
     cudaGraphExec_t graph = nullptr;
@@ -1875,6 +1926,8 @@ static void batch_release(lbm_batch* b) {
         if (t) cudaFree(t);
     if (b->d_flags) cudaFree(b->d_flags);
     if (b->d_maps) cudaFree(b->d_maps);
+    for (int4* t : b->d_march)
+        if (t) cudaFree(t);
     for (cudaEvent_t e : {b->ev_in, b->ev_out, b->ev_fork, b->ev_join, b->t0, b->t1})
         if (e) cudaEventDestroy(e);
     for (int k = 0; k < BATCH_NCLASS; ++k)
@@ -1889,8 +1942,9 @@ static void batch_sync_table(lbm_batch* b) {
     for (int c = 0; c < b->ncases; ++c)
         for (int k = 0; k < BATCH_NCAND; ++k) {
             CaseDesc& d = b->tab(b->cls_of[c], k).c[b->slot_of[c]];
-            if (d.cur != b->cases[c]->cur) {
-                d.cur = b->cases[c]->cur;
+            const int now = b->cases[c]->cur | b->cases[c]->pcur << 1;
+            if (d.cur != now) {
+                d.cur = now;
                 changed = true;
             }
         }
@@ -1912,13 +1966,29 @@ static lbm_status batch_launch(lbm_batch* b, int cls, int cand, int parity) {
     return LBM_OK;
 }
 
-// steps [from, to) of every non-empty class, each class on its own stream
-static lbm_status batch_run(lbm_batch* b, long long from, long long to) {
+// steps [from, to) of every non-empty class, each class on its own stream, with
+// (phi u) in the buffers of parity pp
+static lbm_status batch_run(lbm_batch* b, long long from, long long to, int pp) {
     lbm_status st;
     for (int cls = 0; cls < BATCH_NCLASS; ++cls)
         if (b->ncls[cls])
             for (long long s = from; s < to; ++s)
-                if ((st = batch_launch(b, cls, b->cand[cls], (int)(s & 1))) != LBM_OK) return st;
+                if ((st = batch_launch(b, cls, b->cand[cls], (int)(s & 1) | pp << 1)) != LBM_OK) return st;
+    return LBM_OK;
+}
+
+static bool batch_marches(const lbm_batch* b) { return b->march[0] + b->march[1] > 0; }
+// n pairs of steps of every non-empty class by the two-step kernel, the first
+// reading the buffers of parities 0
+static lbm_status batch_run_pairs(lbm_batch* b, long long n) {
+    for (int cls = 0; cls < BATCH_NCLASS; ++cls)
+        if (b->ncls[cls]) {
+            size_t smem;
+            const MarchBatchKernel k = march_batch_kernel(b->storage, cls, b->check, &smem);
+            for (long long p = 0; p < n; ++p)
+                LBM_BCUDA(b, launch_dep(k, dim3(b->march[cls]), dim3(2 * MARCH_TW), smem, b->bs[cls], b->tab(cls, 0),
+                                        (const int4*)b->d_march[cls], (int)(p & 1) * 3));
+        }
     return LBM_OK;
 }
 
@@ -1949,10 +2019,12 @@ static lbm_status batch_abort(lbm_batch* b, lbm_status st) {
     return st;
 }
 
-// after an odd number of batch steps every case's current buffer flips
-static void batch_flip(lbm_batch* b, long long steps) {
-    if (steps & 1)
-        for (int c = 0; c < b->ncases; ++c) b->cases[c]->cur ^= 1;
+// after an odd number of launches that changed buffers every case's current ones flip
+static void batch_flip(lbm_batch* b, long long flips, long long pflips) {
+    for (int c = 0; c < b->ncases; ++c) {
+        b->cases[c]->cur ^= flips & 1;
+        b->cases[c]->pcur ^= pflips & 1;
+    }
 }
 
 // Time every tile shape of each class on the live state (all shapes give the
@@ -1990,13 +2062,14 @@ static lbm_status batch_tune(lbm_batch* b, long long& done) {
     return LBM_OK;
 }
 
-// Capture BATCH_GRAPH_STEPS steps (parities 0, 1, ...) of both classes, each
+// Capture BATCH_GRAPH_STEPS steps (parities 0, 1, ..., or as many in pairs) of both classes, each
 // class a chain of launches on its own stream, the two chains independent.
 static lbm_status batch_capture(lbm_batch* b) {
     cudaGraph_t g;
     LBM_BCUDA(b, cudaStreamBeginCapture(b->bs[0], cudaStreamCaptureModeThreadLocal));
     lbm_status st = batch_fork(b);
-    if (st == LBM_OK) st = batch_run(b, 0, BATCH_GRAPH_STEPS);
+    if (st == LBM_OK)
+        st = batch_marches(b) ? batch_run_pairs(b, BATCH_GRAPH_STEPS / 2) : batch_run(b, 0, BATCH_GRAPH_STEPS, 0);
     if (st == LBM_OK) st = batch_join(b);
     cudaError_t ce = cudaStreamEndCapture(b->bs[0], &g);
     if (st != LBM_OK) {
@@ -2011,6 +2084,70 @@ static lbm_status batch_capture(lbm_batch* b) {
         return bfail(b, LBM_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(ce));
     }
     return LBM_OK;
+}
+
+// The two-step kernel's block lists of a batch (the classes run side by side):
+// strips as in plan_march, chunks of H rows.  The blocks take H + 7 rows' time
+// each and come in blocks / slots waves and, on average, half a wave of tail; H
+// is the one that makes this least.  us per step of the sweep's first n cases at
+// H = 64 / 96 / 128: FP32 n = 64 309 / 302 / 301, n = 32 163 / 176 / 169, n = 16
+// 83 / 91 / 91; FP16 259 / 256 / 255, 139 / 138 / 144, 73 / 77 / 76.
+// The march is used where every case's grid allows it and the nodes per thread
+// and row time are enough.  One-step kernel -> march (us per step) at shares of
+// 0.72 / 0.66 / 0.56 / 0.45 / 0.43 / 0.32: FP32 391 -> 309, 204 -> 163, 99 -> 83,
+// 43.8 -> 39.9, 26.6 -> 24.0, 8.8 -> 12.1; FP16 275 -> 259, 143 -> 139, 70.7 -> 73.2,
+// 31.9 -> 34.1, 17.3 -> 21.2, 7.6 -> 11.6.  false: out of memory.
+static bool plan_march_batch(lbm_batch* b) {
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device) != cudaSuccess) return true;
+    for (const lbm_handle* h : b->cases)
+        if (h->prm.kernel == LBM_KERNEL_GENERIC || h->nx < 64 || h->ny < 16) return true;
+    const bool fp32 = b->storage == LBM_STORE_FP32;
+    const int slots = sms * (fp32 ? march_minb<ST_FP32>() : march_minb<ST_FP16>());
+    const int most = MARCH_TW - 2 * MARCH_HALO;
+    auto strips = [&](const lbm_handle* h) { return (h->nx + most - 1) / most; };
+    int H = 8;
+    double best = 1e300;
+    for (int k = 8; k <= 256; ++k) {
+        double blocks = 0.0;
+        for (const lbm_handle* h : b->cases) blocks += (double)strips(h) * ((h->ny + k - 1) / k);
+        const double t = (std::fmax(blocks / slots, 0.5) + 0.5) * (k + 7);
+        if (t < best) {
+            best = t;
+            H = k;
+        }
+    }
+    if ((double)b->node_count / ((double)MARCH_TW * slots * best) <
+        (fp32 ? MARCH_BATCH_MIN_SHARE : MARCH_BATCH_MIN_SHARE16))
+        return true;
+    std::vector<int4> list[BATCH_NCLASS];
+    for (int c = 0; c < b->ncases; ++c) {
+        const lbm_handle* h = b->cases[c];
+        const int ns = strips(h), w = (h->nx + ns - 1) / ns, chunks = (h->ny + H - 1) / H;
+        const int rows = (h->ny + chunks - 1) / chunks;
+        for (int k = 0; k * rows < h->ny; ++k)
+            for (int i = 0; i * w < h->nx; ++i) {
+                const int wl = h->nx - i * w < w ? h->nx - i * w : w;
+                const int hl = h->ny - k * rows < rows ? h->ny - k * rows : rows;
+                list[b->cls_of[c]].push_back(make_int4(b->slot_of[c], i * w,
+                                                       (int)((unsigned)(k * rows) | (unsigned)(k & 1) << 31),
+                                                       wl << 16 | hl));
+            }
+    }
+    for (int cls = 0; cls < BATCH_NCLASS; ++cls) {
+        if (list[cls].empty()) continue;
+        size_t smem;
+        const MarchBatchKernel k = march_batch_kernel(b->storage, cls, b->check, &smem);
+        const size_t bytes = list[cls].size() * sizeof(int4);
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+            cudaMalloc(&b->d_march[cls], bytes) != cudaSuccess ||
+            cudaMemcpy(b->d_march[cls], list[cls].data(), bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
+            bfail(b, LBM_ERR_OOM, "block list allocation failed");
+            return false;
+        }
+    }
+    for (int cls = 0; cls < BATCH_NCLASS; ++cls) b->march[cls] = (int)list[cls].size();
+    return true;
 }
 
 extern "C" {
@@ -2102,7 +2239,7 @@ lbm_status lbm_batch_create(int ncases, lbm_handle* const* cases, lbm_batch** ou
                 d.flag = h->flag;
                 d.nx = h->nx;
                 d.ny = h->ny;
-                d.cur = h->cur;
+                d.cur = h->cur | h->pcur << 1;
                 d.map0 = -1;
                 d.m = h->model;
                 tiles += (long long)((h->nx + BATCH_TX[k] - 1) / BATCH_TX[k]) * ((h->ny + th - 1) / th);
@@ -2158,8 +2295,8 @@ lbm_status lbm_batch_create(int ncases, lbm_handle* const* cases, lbm_batch** ou
                 std::vector<CUtensorMap> maps((size_t)ncases * 8);
                 bool ok = true;
                 for (int c = 0; c < ncases && ok; ++c)
-                    ok = encode_maps16(cases[c], 0, &maps[8 * c], BATCH_PF_BOX_X, BATCH_PF_BOX_Y) &&
-                         encode_maps16(cases[c], 1, &maps[8 * c + 4], BATCH_PF_BOX_X, BATCH_PF_BOX_Y);
+                    ok = encode_maps16(cases[c], 0, cases[c]->pcur, &maps[8 * c], BATCH_PF_BOX_X, BATCH_PF_BOX_Y) &&
+                         encode_maps16(cases[c], 1, cases[c]->pcur, &maps[8 * c + 4], BATCH_PF_BOX_X, BATCH_PF_BOX_Y);
                 if (ok && cudaMalloc(&b->d_maps, maps.size() * sizeof(CUtensorMap)) == cudaSuccess &&
                     cudaMemcpy(b->d_maps, maps.data(), maps.size() * sizeof(CUtensorMap),
                                cudaMemcpyHostToDevice) == cudaSuccess) {
@@ -2177,6 +2314,7 @@ lbm_status lbm_batch_create(int ncases, lbm_handle* const* cases, lbm_batch** ou
             }
         }
     }
+    if (!plan_march_batch(b)) return bad(LBM_ERR_OOM);
     // batch index of each class slot, for gathering the cases' flags
     for (int cls = 0; cls < BATCH_NCLASS; ++cls) {
         if (!b->ncls[cls]) continue;
@@ -2245,7 +2383,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps) {
         if ((st = batch_tune(b, done)) != LBM_OK) return batch_abort(b, st);
     // an odd count so far: one more step so the graph starts at parity 0
     if ((done & 1) && done < nsteps) {
-        if ((st = batch_run(b, done, done + 1)) != LBM_OK) return batch_abort(b, st);
+        if ((st = batch_run(b, done, done + 1, 0)) != LBM_OK) return batch_abort(b, st);
         ++done;
     }
     if ((st = batch_join(b)) != LBM_OK) return batch_abort(b, st);
@@ -2260,15 +2398,25 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps) {
                                             cudaGetErrorString(ce)));
         }
     }
-    // the remainder, with parities continuing from 0 after the replays
-    if (done + reps * BATCH_GRAPH_STEPS < nsteps) {
+    // the remainder, with parities continuing from 0 after the replays; flips: the
+    // launches that changed buffers since the parity was 0
+    const long long at = done + reps * BATCH_GRAPH_STEPS, rest = nsteps - at;
+    long long flips = done + rest, pflips = 0;
+    if (rest > 0) {
         if ((st = batch_fork(b)) != LBM_OK) return batch_abort(b, st);
-        if ((st = batch_run(b, done + reps * BATCH_GRAPH_STEPS, nsteps)) != LBM_OK)
+        if (batch_marches(b)) {
+            pflips = rest / 2;  // (here `done` is even)
+            flips = pflips + (rest & 1);
+            if ((st = batch_run_pairs(b, pflips)) != LBM_OK) return batch_abort(b, st);
+            if ((rest & 1) && (st = batch_run(b, pflips, pflips + 1, (int)(pflips & 1))) != LBM_OK)
+                return batch_abort(b, st);
+        } else if ((st = batch_run(b, at, nsteps, 0)) != LBM_OK) {
             return batch_abort(b, st);
+        }
         if ((st = batch_join(b)) != LBM_OK) return batch_abort(b, st);
     }
     // cases' current buffers (and with them the tables) follow
-    batch_flip(b, nsteps);
+    batch_flip(b, flips, pflips);
     batch_sync_table(b);
     if (b->check) {
         // the cases' non-finite flags (set by any step of this call), gathered

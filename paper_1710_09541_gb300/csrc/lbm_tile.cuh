@@ -65,7 +65,7 @@ __device__ __forceinline__ void tile_block(char* smem, const MarchArgs& A, const
             R = Row{};
         } else
 #endif
-            R.template pull<W>(A.s, o, lo, hi);
+            R.template pull<W>(A, o, lo, hi);
     }
     // neighbours in shared memory, as byte offsets from the own slot: rows w1 apart;
     // at the open top the row above is the row itself, at an edge row the ghost
@@ -95,7 +95,7 @@ __device__ __forceinline__ void tile_block(char* smem, const MarchArgs& A, const
             if (s < S)
                 Row::template put_ring<LP>(own, f, g, phi, pu, (unsigned)(y * nx + x), seed);
             else
-                Row::put(A.d, 4u * (y * nx + x), f, g, phi, pu, seed);
+                Row::put(A, 4u * (y * nx + x), f, g, phi, pu, seed);
         }
         __syncthreads();
     }

@@ -92,3 +92,33 @@ def test_march_in_the_checking_build(libs, storage):
             lbm._LIB_PATH, lbm._lib = path, None
             got.append(_run(lbm, nx, ny, bc, storage, (9,), 0, 0, 3))
         _same(*got)
+
+
+def _batch(lbm, n, storage, kernel, steps, check_every=0):
+    specs = cases.batch_cases(n, seed=11)
+    specs[3]["params"] = dict(specs[3]["params"], bc_y=2)
+    lats = [lbm.Lattice(sp["nx"], sp["ny"], storage=storage, kernel=kernel, check_every=check_every, **sp["params"])
+            .init(sp["phi0"], sp["ux0"], sp["uy0"]) for sp in specs]
+    try:
+        with lbm.Batch(lats) as bt:
+            for k in steps:
+                bt.step(k)
+                lats[2].step(3)  # a case stepped on its own in between
+        return [a for lat in lats for a in lat.get_state()]
+    finally:
+        for lat in lats:
+            lat.close()
+
+
+@pytest.mark.parametrize("n,storage,check_every", [(16, 0, 0), (16, 0, 1), (36, 1, 0), (36, 2, 2)])
+def test_batch_march_equals_single_steps(libs, n, storage, check_every):
+    """Batches large enough to march: fewer steps than a graph, odd counts, the
+    tuning call, graph replays with even and odd remainders."""
+    lbm, release, debug = libs
+    steps = (7, 4, 1, 151, 67, 34)
+    lbm._LIB_PATH, lbm._lib = release, None
+    got = _batch(lbm, n, storage, 0, steps, check_every)
+    _same(got, _batch(lbm, n, storage, 1, steps, check_every))
+    if check_every:
+        lbm._LIB_PATH, lbm._lib = debug, None
+        _same(_batch(lbm, n, storage, 0, steps, check_every), got)
