@@ -132,7 +132,8 @@ __device__ __forceinline__ bool nbr_in_range(const Nbr& q, int nx, int ny) {
 #endif
 // One TX x TY tile with origin (x0, y0): the body shared by the single-case
 // step kernel and the batched kernel (so both give the same bits).
-template <int TX, int TY, bool FIELDS, int WALLS, int ST, bool CHK>
+// PK: packed arithmetic (F2).
+template <int TX, int TY, bool FIELDS, int WALLS, int ST, bool CHK, bool PK = false>
 __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __restrict__ fs,
                                           const float* __restrict__ gs, float* __restrict__ fd,
                                           float* __restrict__ gd, float* __restrict__ phiu,
@@ -196,10 +197,10 @@ __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __
 
     const int lx = tx + 1, ly = ty + 1;
     const float phi = sphi[ly][lx];
-    const Stencil st = stencil(phi, sphi[ly][lx + 1], sphi[ly][lx - 1], sphi[ly + 1][lx],
+    const Stencil st = stencil<PK>(phi, sphi[ly][lx + 1], sphi[ly][lx - 1], sphi[ly + 1][lx],
                                sphi[ly - 1][lx], sphi[ly + 1][lx + 1], sphi[ly + 1][lx - 1],
                                sphi[ly - 1][lx - 1], sphi[ly - 1][lx + 1]);
-    const Macro M = macro_from(m, Pop<ST>::gmom(g), phi, st.gx, st.gy, st.lap);
+    const Macro M = macro_from<PK>(m, Pop<ST>::template gmom<PK>(g), phi, st.gx, st.gy, st.lap);
     const int n32 = q.r0 + x;
 
     if (FIELDS) {
@@ -218,7 +219,7 @@ __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __
 #if !LBM_EARLY_PHIU
     const float2 prev = make_float2(phiu[n32], phiu[N32 + n32]);
 #endif
-    const float2 now = collide_st<ST>(m, f, g, phi, st, M, prev);
+    const float2 now = collide_st<ST, PK>(m, f, g, phi, st, M, prev);
     phiu[n32] = now.x;
     phiu[N32 + n32] = now.y;
     Pop<ST>::stfg(fd, gd, N32, n32, f, g, phi);
@@ -243,6 +244,11 @@ __device__ __forceinline__ void step_tile16(float (*sphi)[TX + 2], const void* _
                                             int x0, int y0) {
     constexpr bool BR = (WALLS < 0) || LBM_WALL_BRANCH;
     constexpr int TH = TY * NPT;
+    // Packed arithmetic (F2): the 16-bit step is bound by instruction issue.  us per
+    // step, scalar -> packed: FP16 768^2 10.6 -> 10.3, 1024^2 18.4 -> 17.4, 2048^2 71.3 ->
+    // 64.6, walled 800 x 500 8.4 -> 7.8, 2400 x 600 25.8 -> 24.4, 64-case batch 276 -> 264;
+    // BF16 2048^2 73.4 -> 65.9, batch 283 -> 267; BF16-SR 2048^2 73.6 -> 68.6.
+    constexpr bool PK = true;
     if (WALLS == 0) m.walls = 0;  // WALLS == 1 keeps the kind of top (wall or open)
     const int wfold = WALLS >= 0 ? WALLS : m.walls;  // y folding: wrap (0) or clamp
     const int N = nx * ny;  // 20 N < 2^31 (checked at create): 32-bit offsets
@@ -278,7 +284,7 @@ __device__ __forceinline__ void step_tile16(float (*sphi)[TX + 2], const void* _
             pull_words16<ST, BR, true>(fs, gs, N, q, w[j], f0[j], g0[j]);
             float h[9];
             codes_f<ST>(w[j], f0[j], h);
-            sphi[ly + 1][tx + 1] = Pop<ST>::phi_of(h);
+            sphi[ly + 1][tx + 1] = Pop<ST>::template phi_of<PK>(h);
         } else {
             sphi[ly + 1][tx + 1] =
                 phi_at_st<ST, WALLS>(fs, N, fold_x(x, nx), fold_y(y, ny, wfold), nx, ny, m.walls);
@@ -306,16 +312,16 @@ __device__ __forceinline__ void step_tile16(float (*sphi)[TX + 2], const void* _
         codes_f<ST>(w[j], f0[j], h);
         codes_g<ST>(w[j], g0[j], k);
         const float phi = sphi[ly][lx];
-        const Stencil st = stencil(phi, sphi[ly][lx + 1], sphi[ly][lx - 1], sphi[ly + 1][lx],
+        const Stencil st = stencil<PK>(phi, sphi[ly][lx + 1], sphi[ly][lx - 1], sphi[ly + 1][lx],
                                    sphi[ly - 1][lx], sphi[ly + 1][lx + 1], sphi[ly + 1][lx - 1],
                                    sphi[ly - 1][lx - 1], sphi[ly - 1][lx + 1]);
-        const Macro M = macro_from(m, Pop<ST>::gmom(k), phi, st.gx, st.gy, st.lap);
+        const Macro M = macro_from<PK>(m, Pop<ST>::template gmom<PK>(k), phi, st.gx, st.gy, st.lap);
         bool bad = false;
         if constexpr (CHK) bad = m.check_nonfinite && !isfinite(add(add(phi, M.ux), add(M.uy, M.p)));
-        const float2 now = collide_code<Pop<ST>>(m, h, k, phi, st, M, prev[j]);
+        const float2 now = collide_code<Pop<ST>, PK>(m, h, k, phi, st, M, prev[j]);
         phiu[n[j]] = now.x;
         phiu[N + n[j]] = now.y;
-        Pop<ST>::stfg(fd, gd, N, n[j], h, k, phi, m.seed);
+        Pop<ST>::template stfg<PK>(fd, gd, N, n[j], h, k, phi, m.seed);
         if constexpr (CHK)
             if (bad) report_nonfinite(flag);
     }
@@ -421,7 +427,7 @@ __device__ __forceinline__ void prefetch_tile(const void* fs, const void* gs, co
 #ifndef LBM_MARCH_THREADS16
 #define LBM_MARCH_THREADS16 768
 #endif
-constexpr double MARCH_BATCH_MIN_SHARE = 0.40, MARCH_BATCH_MIN_SHARE16 = 0.62;  // see plan_march_batch
+constexpr double MARCH_BATCH_MIN_SHARE = 0.40, MARCH_BATCH_MIN_SHARE16 = 0.70;  // see plan_march_batch
 // Resident blocks per SM each step kernel is compiled for (its register
 // budget), measured per instantiation with 32 x 4 tiles at 2048^2 (2400 x 600
 // for walls), MLUPS at 8 / 9 / 10 blocks:
@@ -447,7 +453,7 @@ __host__ __device__ constexpr int step_npt() {
     return (!FIELDS && ST != ST_FP32) ? LBM_NPT16 : 1;
 }
 
-template <int TX, int TY, bool FIELDS, int WALLS, int ST, bool CHK = false>
+template <int TX, int TY, bool FIELDS, int WALLS, int ST, bool CHK = false, bool PK = false>
 __global__ void __launch_bounds__(TX* TY, (step_minb<FIELDS, WALLS, ST, TX * TY>()))
     k_step(const float* __restrict__ fs, const float* __restrict__ gs, float* __restrict__ fd,
            float* __restrict__ gd, float* __restrict__ phiu, unsigned int* __restrict__ flag,
@@ -483,7 +489,7 @@ __global__ void __launch_bounds__(TX* TY, (step_minb<FIELDS, WALLS, ST, TX * TY>
         step_tile16<TX, TY, NPT, WALLS, ST, CHK>(sphi, fs, gs, fd, gd, phiu, flag, nx, ny, m,
                                                  bx * TX, by * TY * NPT);
     else
-        step_tile<TX, TY, FIELDS, WALLS, ST, CHK>(sphi, fs, gs, fd, gd, phiu, flag, out, nx, ny, m,
+        step_tile<TX, TY, FIELDS, WALLS, ST, CHK, PK>(sphi, fs, gs, fd, gd, phiu, flag, out, nx, ny, m,
                                                   bx * TX, by * TY);
 }
 
@@ -956,7 +962,17 @@ static lbm_status launch_step(lbm_handle* h, bool fields, double* out) {
         case LBM_STORE_BF16_SHIFTED_SR:
             k = fields ? LBM_STEP_KERNEL(ST_BF16, STEP16_TX) : LBM_STEP_KERNEL(ST_BF16_SR, STEP16_TX);
             break;
-        default: k = LBM_STEP_KERNEL(ST_FP32, STEP_TX);
+        default:
+            // FP32 grids whose step stays in L2 are not bound by DRAM, and take the
+            // packed arithmetic: 256^2 3.36 -> 3.18 us, 384^2 5.08 -> 4.58, 512^2 6.75
+            // -> 6.51, 1024^2 26.5 -> 25.7.  Larger ones lose by it: 1152^2 34.1 ->
+            // 35.0, walled 1600 x 800 34.9 -> 35.7, 1501 x 1103 50.7 -> 51.5.
+            k = LBM_STEP_KERNEL(ST_FP32, STEP_TX);
+            if (!fields && h->pf_ahead == 0)
+                k = walls ? (chk ? k_step<STEP_TX, STEP_TY, false, 1, ST_FP32, true, true>
+                                 : k_step<STEP_TX, STEP_TY, false, 1, ST_FP32, false, true>)
+                          : (chk ? k_step<STEP_TX, STEP_TY, false, 0, ST_FP32, true, true>
+                                 : k_step<STEP_TX, STEP_TY, false, 0, ST_FP32, false, true>);
     }
 #undef LBM_STEP_KERNEL
     if (fields)
@@ -998,12 +1014,12 @@ static MarchKernel march_kernel(const lbm_params& p, size_t* smem) {
 // Strips and chunks of a handle's two-step launches: one resident wave of
 // blocks.  A block computes TW columns for w of its own and takes about H + 7
 // rows' time for H, so the march pays where eff = w / TW * H / (H + 7) is high
-// enough.  One-step time / march time at eff, nx a multiple of 8: FP32 640 x 400
-// 0.39 0.92, 560^2 0.44 1.02, 704^2 0.54 1.09, 1000 x 600 0.55 1.26, 960^2 0.66
-// 1.46; FP16 800 x 500 0.48 0.97, 768^2 0.54 0.95, 1000 x 600 0.55 1.03, 960^2 0.66
-// 1.07.  Other nx, whose rows start inside a 32-byte sector, slow the one-step
-// kernels down: FP32 501^2 0.36 1.13, 901 x 300 0.41 1.18; FP16 901 x 300 0.41 0.99,
-// 601^2 0.47 1.19.
+// enough.  One-step time / march time at eff, nx a multiple of 8: FP32 640^2 0.47
+// 0.94, 768^2 0.54 1.09, 896^2 0.61 1.29, 1024^2 0.67 1.32; FP16 896^2 0.61 0.95, 1024^2
+// 0.67 0.98, 1152^2 0.71 1.05, 1280^2 0.75 1.10, walled 800 x 500 0.48 0.92, 1200 x 700
+// 0.65 1.04, 2400 x 600 0.75 1.08.  Other nx, whose rows start inside a 32-byte sector,
+// slow the one-step kernels down: FP32 501^2 0.36 1.14, 901 x 300 0.41 1.17; FP16 901 x
+// 300 0.41 0.97, 601^2 0.47 1.14, 801^2 0.58 1.10, 1001^2 0.66 1.01, 1501 x 1103 0.74 1.15.
 static MarchGrid plan_march(int nx, int ny, const lbm_params& p, int sms) {
     MarchGrid g = {0, 0, 0};
     if (p.kernel == LBM_KERNEL_GENERIC || nx < 64 || ny < 16) return g;
@@ -1015,7 +1031,7 @@ static MarchGrid plan_march(int nx, int ny, const lbm_params& p, int sms) {
     g.H = (ny + chunks - 1) / chunks;
     const double eff = (double)g.w / MARCH_TW * g.H / (g.H + 7);
     const bool fp32 = p.storage == LBM_STORE_FP32;
-    if (eff < (nx % 8 == 0 ? (fp32 ? 0.43 : 0.55) : (fp32 ? 0.36 : 0.42))) g.H = 0;
+    if (eff < (nx % 8 == 0 ? (fp32 ? 0.50 : p.bc_y != LBM_BC_PERIODIC ? 0.62 : 0.69) : (fp32 ? 0.36 : 0.42))) g.H = 0;
     return g;
 }
 
@@ -2095,8 +2111,8 @@ static lbm_status batch_capture(lbm_batch* b) {
 // The march is used where every case's grid allows it and the nodes per thread
 // and row time are enough.  One-step kernel -> march (us per step) at shares of
 // 0.72 / 0.66 / 0.56 / 0.45 / 0.43 / 0.32: FP32 391 -> 309, 204 -> 163, 99 -> 83,
-// 43.8 -> 39.9, 26.6 -> 24.0, 8.8 -> 12.1; FP16 275 -> 259, 143 -> 139, 70.7 -> 73.2,
-// 31.9 -> 34.1, 17.3 -> 21.2, 7.6 -> 11.6.  false: out of memory.
+// 43.8 -> 39.9, 26.6 -> 24.0, 8.8 -> 12.1; FP16 263 -> 256, 137 -> 139, 67 -> 73,
+// 30.6 -> 34.1, 15.9 -> 21.2, 7.4 -> 11.6.  false: out of memory.
 static bool plan_march_batch(lbm_batch* b) {
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->device) != cudaSuccess) return true;

@@ -293,13 +293,14 @@ struct Shifted16 {
         f0 = sub(phi, s8<PK>(d));
     }
     // store the post-collision codes of node idx
+    template <bool PK = false>
     __device__ static void stfg(void* fb, void* gb, int N, int idx, const float h[9],
                                 const float k[9], float phi, unsigned int seed = 0) {
         unsigned int* P = pw(fb, N);
         unsigned int w[9];
         float f0;
         unsigned short k0;
-        encode(h, k, phi, (unsigned int)idx, seed, w, f0, k0);
+        encode<PK>(h, k, phi, (unsigned int)idx, seed, w, f0, k0);
 #pragma unroll
         for (int i = 1; i < 9; ++i) P[(i - 1) * N + idx] = w[i];
         static_cast<float*>(fb)[idx] = f0;
