@@ -130,6 +130,10 @@ __device__ __forceinline__ bool nbr_in_range(const Nbr& q, int nx, int ny) {
 #ifndef LBM_PREFETCH16_TMA_L2X10
 #define LBM_PREFETCH16_TMA_L2X10 15
 #endif
+// Where a read-back writes phi, rho, ux, uy, p (N doubles each; nullptr: not wanted).
+struct FieldsOut {
+    double* p[5];
+};
 // One TX x TY tile with origin (x0, y0): the body shared by the single-case
 // step kernel and the batched kernel (so both give the same bits).
 // PK: packed arithmetic (F2).
@@ -137,7 +141,7 @@ template <int TX, int TY, bool FIELDS, int WALLS, int ST, bool CHK, bool PK = fa
 __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __restrict__ fs,
                                           const float* __restrict__ gs, float* __restrict__ fd,
                                           float* __restrict__ gd, float* __restrict__ phiu,
-                                          unsigned int* __restrict__ flag, double* __restrict__ out,
+                                          unsigned int* __restrict__ flag, const FieldsOut& out,
                                           int nx, int ny, Model m, int x0, int y0) {
     if (WALLS == 0) m.walls = 0;  // WALLS == 1 keeps the kind of top (wall or open)
     const int wfold = WALLS >= 0 ? WALLS : m.walls;  // y folding: wrap (0) or clamp
@@ -204,11 +208,10 @@ __device__ __forceinline__ void step_tile(float (*sphi)[TX + 2], const float* __
     const int n32 = q.r0 + x;
 
     if (FIELDS) {
-        out[n32] = phi;
-        out[N + n32] = M.rho;
-        out[2 * N + n32] = M.ux;
-        out[3 * N + n32] = M.uy;
-        out[4 * N + n32] = M.p;
+        const float v[5] = {phi, M.rho, M.ux, M.uy, M.p};
+#pragma unroll
+        for (int k = 0; k < 5; ++k)
+            if (out.p[k]) out.p[k][n32] = v[k];
         return;
     }
     // one test: a NaN or Inf in any of phi, u, p makes the sum non-finite;
@@ -457,7 +460,7 @@ template <int TX, int TY, bool FIELDS, int WALLS, int ST, bool CHK = false, bool
 __global__ void __launch_bounds__(TX* TY, (step_minb<FIELDS, WALLS, ST, TX * TY>()))
     k_step(const float* __restrict__ fs, const float* __restrict__ gs, float* __restrict__ fd,
            float* __restrict__ gd, float* __restrict__ phiu, unsigned int* __restrict__ flag,
-           double* __restrict__ out, int nx, int ny, Model m, int pf_ahead, int rev,
+           const __grid_constant__ FieldsOut out, int nx, int ny, Model m, int pf_ahead, int rev,
            const __grid_constant__ PfMaps pm) {
     constexpr int NPT = step_npt<FIELDS, ST>();
     __shared__ float sphi[TY * NPT + 2][TX + 2];
@@ -934,7 +937,7 @@ static cudaError_t launch_dep(void (*k)(Exp...), dim3 grid, dim3 block, size_t s
     return cudaLaunchKernelEx(&cfg, k, std::forward<Act>(args)...);
 }
 
-static lbm_status launch_step(lbm_handle* h, bool fields, double* out) {
+static lbm_status launch_step(lbm_handle* h, bool fields, const FieldsOut& out = FieldsOut{}) {
     const int c = h->cur;
     const bool walls = h->model.walls != 0;
     // a 16-bit step's thread takes LBM_NPT16 nodes, so its tile is that many times taller
@@ -943,7 +946,7 @@ static lbm_status launch_step(lbm_handle* h, bool fields, double* out) {
     const int th = st16 ? STEP_TY * LBM_NPT16 : STEP_TY;
     dim3 block(tw, STEP_TY);
     dim3 grid((h->nx + tw - 1) / tw, (h->ny + th - 1) / th);
-    using K = void (*)(const float*, const float*, float*, float*, float*, unsigned int*, double*,
+    using K = void (*)(const float*, const float*, float*, float*, float*, unsigned int*, FieldsOut,
                        int, int, Model, int, int, PfMaps);
     K k;
     // the steps of a handle that asked for non-finite checks test every node;
@@ -985,7 +988,7 @@ static lbm_status launch_step(lbm_handle* h, bool fields, double* out) {
         h->model.seed = (unsigned int)(++h->nstep) * 0x9e3779b9u;
         LBM_CUDA(h, launch_dep(k, grid, block, 0, h->stream, (const float*)h->f[c],
                                (const float*)h->g[c], h->f[c ^ 1], h->g[c ^ 1], h->phiu[h->pcur], h->flag,
-                               (double*)nullptr, h->nx, h->ny, h->model, h->pf_ahead,
+                               FieldsOut{}, h->nx, h->ny, h->model, h->pf_ahead,
                                LBM_ALTERNATE_ORDER ? c : 0, pm));
     }
     LBM_CUDA(h, cudaGetLastError());
@@ -1144,6 +1147,63 @@ static lbm_status check_flag(lbm_handle* h) {
         return fail(h, LBM_ERR_NONFINITE, "non-finite phi, u or p produced by a step");
     }
     return LBM_OK;
+}
+
+constexpr size_t DIRECT_SMALL = 150000;  // nodes
+// the five planes in the staging buffer
+static FieldsOut staged_fields(const lbm_handle* h) {
+    FieldsOut o;
+    for (int k = 0; k < 5; ++k) o.p[k] = (double*)h->staging + k * h->N;
+    return o;
+}
+
+// Whether every wanted output lies whole in one page-locked, device-mapped host
+// allocation: then the read-back kernel writes them itself, over the link to the
+// host, instead of writing the staging buffer for five copies to read.  Any other
+// memory takes the copies.
+// Rows that start inside a 64-byte line are written in pieces, which pays only
+// where the calls cost more than the bytes.  us per read-back, copies -> kernel:
+// 64^2 34 -> 25, 301 x 300 52 -> 46, 501 x 400 77 -> 77, 1501 x 1103 413 -> 464; whole
+// lines: 256^2 46 -> 37, 1024^2 275 -> 240, 2048^2 987 -> 892.
+static bool pinned_outputs(double* const outs[5], int nx, size_t nodes, FieldsOut* o) {
+    const size_t bytes = nodes * sizeof(double);
+    const bool small = nodes <= DIRECT_SMALL;
+    if (nx % 8 != 0 && !small) return false;
+    static PFN_cuPointerGetAttribute_v4000 get = nullptr;
+    static std::once_flag once;
+    std::call_once(once, [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &f, 4000, cudaEnableDefault, &q) ==
+                cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            get = (PFN_cuPointerGetAttribute_v4000)f;
+    });
+    if (!get) return false;
+    for (int k = 0; k < 5; ++k) {
+        o->p[k] = nullptr;
+        if (!outs[k]) continue;
+        for (int j = 0; j < k; ++j) {  // overlapping outputs take the copies, whose order decides
+            const uintptr_t a = (uintptr_t)outs[j], b = (uintptr_t)outs[k];
+            if (outs[j] && (a > b ? a - b : b - a) < bytes) return false;
+        }
+        cudaPointerAttributes at{};
+        if (cudaPointerGetAttributes(&at, outs[k]) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        CUdeviceptr start = 0;
+        size_t size = 0;
+        if (at.type != cudaMemoryTypeHost || !at.devicePointer ||
+            get(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)outs[k]) != CUDA_SUCCESS ||
+            get(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, (CUdeviceptr)outs[k]) != CUDA_SUCCESS)
+            return false;
+        const size_t at_byte = (size_t)((uintptr_t)outs[k] - (uintptr_t)start);
+        if ((uintptr_t)outs[k] < (uintptr_t)start || at_byte + bytes > size || (uintptr_t)at.devicePointer % (small ? 8 : 64) != 0)
+            return false;
+        o->p[k] = (double*)at.devicePointer;
+    }
+    return true;
 }
 
 extern "C" {
@@ -1414,7 +1474,7 @@ lbm_status lbm_step(lbm_handle* h, int nsteps) {
         if (h->prm.check_every > 0 && h->prm.check_every - h->since_check < n)
             n = (int)(h->prm.check_every - h->since_check);
         n = h->tile.S > 1 ? (n < h->tile.S ? n : h->tile.S) : h->march.H > 0 && n > 1 ? 2 : 1;
-        lbm_status st = n == 1 ? launch_step(h, false, nullptr) : h->tile.S > 1 ? launch_tile(h, n) : launch_march(h);
+        lbm_status st = n == 1 ? launch_step(h, false) : h->tile.S > 1 ? launch_tile(h, n) : launch_march(h);
         if (st != LBM_OK) return st;
         s += n;
         if (h->prm.check_every > 0 && (h->since_check += n) >= h->prm.check_every) {
@@ -1430,14 +1490,20 @@ lbm_status lbm_get_fields(lbm_handle* h, double* phi, double* rho, double* ux, d
     if (!h) return LBM_ERR_INVALID;
     if (!h->inited) return fail(h, LBM_ERR_STATE, "lbm_get_fields before lbm_init");
     LBM_CUDA(h, cudaSetDevice(h->device));
-    double* buf = (double*)h->staging;
-    lbm_status st = launch_step(h, true, buf);
-    if (st != LBM_OK) return st;
     double* outs[5] = {phi, rho, ux, uy, p};
-    for (int k = 0; k < 5; ++k)
-        if (outs[k])
-            LBM_CUDA(h, cudaMemcpyAsync(outs[k], buf + k * h->N, h->N * sizeof(double),
-                                        cudaMemcpyDeviceToHost, h->stream));
+    FieldsOut direct;
+    if (pinned_outputs(outs, h->nx, h->N, &direct)) {
+        lbm_status st = launch_step(h, true, direct);
+        if (st != LBM_OK) return st;
+    } else {
+        double* buf = (double*)h->staging;
+        lbm_status st = launch_step(h, true, staged_fields(h));
+        if (st != LBM_OK) return st;
+        for (int k = 0; k < 5; ++k)
+            if (outs[k])
+                LBM_CUDA(h, cudaMemcpyAsync(outs[k], buf + k * h->N, h->N * sizeof(double),
+                                            cudaMemcpyDeviceToHost, h->stream));
+    }
     LBM_CUDA(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }
@@ -1488,7 +1554,7 @@ lbm_status lbm_diag(lbm_handle* h, double* sum_phi, double* umax, double* pmin, 
     if (!h->inited) return fail(h, LBM_ERR_STATE, "lbm_diag before lbm_init");
     LBM_CUDA(h, cudaSetDevice(h->device));
     double* buf = (double*)h->staging;
-    lbm_status st = launch_step(h, true, buf);
+    lbm_status st = launch_step(h, true, staged_fields(h));
     if (st != LBM_OK) return st;
     k_diag_partial<<<RED_BLOCKS, RED_THREADS, 0, h->stream>>>(buf, h->N, h->red_part);
     LBM_CUDA(h, cudaGetLastError());
@@ -1783,7 +1849,7 @@ __global__ void __launch_bounds__(TX* TY, (ST == ST_FP32 ? LBM_BATCH_THREADS : L
     float* const pu = cd.phiu[((cd.cur >> 1) + (parity >> 1)) & 1];
     if constexpr (ST == ST_FP32) {
         step_tile<TX, TY, false, WALLS, ST, CHK>(sphi, cd.f[c], cd.g[c], cd.f[c ^ 1], cd.g[c ^ 1], pu,
-                                                 cd.flag, nullptr, cd.nx, cd.ny, cd.m, (e.y & 0xffff) * TX,
+                                                 cd.flag, FieldsOut{}, cd.nx, cd.ny, cd.m, (e.y & 0xffff) * TX,
                                             (e.y >> 16) * TY);
     } else {
         step_tile16<TX, TY, LBM_NPT16_BATCH, WALLS, ST, CHK>(
@@ -2623,7 +2689,7 @@ lbm_status lbm_laplace_jump(lbm_handle* h, double xc, double yc, double r_in, do
         return fail(h, LBM_ERR_INVALID, "lbm_laplace_jump: need finite centre and 0 < r_in <= r_out");
     LBM_CUDA(h, cudaSetDevice(h->device));
     double* buf = (double*)h->staging;
-    lbm_status st = launch_step(h, true, buf);
+    lbm_status st = launch_step(h, true, staged_fields(h));
     if (st != LBM_OK) return st;
     k_jump_partial<<<RED_BLOCKS, RED_THREADS, 0, h->stream>>>(buf, h->nx, h->ny, h->model.walls == 0,
                                                                xc, yc, r_in * r_in, r_out * r_out,
