@@ -1086,14 +1086,19 @@ static TileGrid plan_tile(int nx, int ny, const lbm_params& p, int sms) {
     const double n = (double)nx * ny;
     if (p.kernel == LBM_KERNEL_GENERIC || n > 1e5) return best;
     double t = 0.95 * (p.storage == LBM_STORE_FP32 ? 2.45 + 1.5e-5 * n : 3.0 + 0.9e-5 * n);
+    int cols[33], rows[33];  // tiles of width / height k across the grid
+    for (int k = 2; k <= 32; ++k) {
+        cols[k] = (nx + k - 1) / k;
+        rows[k] = (ny + k - 1) / k;
+    }
     for (int S = 2; S <= 6; ++S)
         for (int h = 2; h <= 32 && h <= ny; ++h)
-            for (int w = 2; w <= 32 && w <= nx; ++w) {
-                if ((w + 4 * S - 2) * (h + 4 * S - 2) > TILE_THREADS) continue;
-                int nodes = 0;
-                for (int s = 1; s <= S; ++s) nodes += (w + 4 * (S - s) + 2) * (h + 4 * (S - s) + 2);
-                const int blocks = ((nx + w - 1) / w) * ((ny + h - 1) / h);
-                const double us = (1.78 + 2.8e-3 * nodes * ((blocks + sms - 1) / sms)) / S;
+            for (int w = 2; w <= 32 && w <= nx && (w + 4 * S - 2) * (h + 4 * S - 2) <= TILE_THREADS; ++w) {
+                // sum over j = 0 .. S-1 of (w + 2 + 4 j) (h + 2 + 4 j)
+                const int nodes = S * (w + 2) * (h + 2) + 2 * S * (S - 1) * (w + h + 4) +
+                                  8 * S * (S - 1) * (2 * S - 1) / 3;
+                const int waves = (cols[w] * rows[h] + sms - 1) / sms;
+                const double us = (1.78 + 2.8e-3 * nodes * waves) / S;
                 if (us < t) {
                     t = us;
                     best = TileGrid{w, h, S};
