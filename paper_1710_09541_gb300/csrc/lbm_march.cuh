@@ -30,17 +30,21 @@
 // theirs bit for bit.
 //
 // What bounds it: latency.  At 2048^2 with FP32 storage a launch (two steps)
-// moves 622 MB, 0.64 of the measured copy bandwidth, at an IPC of about 2 of 4.
-// Measured (us per step at 2048^2, one-step kernel -> this one): FP32 103.2 ->
-// 70.9, FP16 70.4 -> 58.5, BF16-SR 73.6 -> 61.1; at 1501 x 1103 51.9 -> 29.8,
-// 32.2 -> 25.6, 33.6 -> 26.7; walled 2400 x 600 39.6 -> 26.7, 26.5 -> 22.9,
-// 27.4 -> 23.9.  One set of threads taking both steps, with four blocks of 128
-// threads per SM, took 84.5 (FP32) and 59.0 (FP16): its 112 registers left 16
-// warps to cover the loads.  Three blocks of 2 x 128 threads at 80 registers
-// beat two at 128 (82.3 / 69.8) and four at 64 (spills: 86.7 / 62.4); strips of
-// 64 / 96 / 192 threads 71.9 / 72.7 / 75.5 against 71.2 at 128.
-// L2 prefetch of the rows ahead (bulk copies or tensor boxes) made it slower at
-// every distance above one row and was left out.
+// moves 620 MB of DRAM traffic in 139 us, 0.66 of the measured copy bandwidth, at
+// an IPC of 2.1 of 4; with FP16 335 MB at an IPC of 2.6.
+// Measured (us per step, one-step kernel of its time -> this one): FP32 2048^2
+// 103.2 -> 69.6, 1501 x 1103 51.9 -> 29.4, walled 2400 x 600 39.6 -> 26.6; FP16 70.4
+// (64.6 with packed arithmetic) -> 59.4, 32.2 -> 25.7, 26.5 (24.4) -> 22.8; BF16-SR
+// 73.6 (68.6) -> 62.3, 33.6 -> 27.0, 27.4 (25.2) -> 23.8.  One set of threads taking
+// both steps, with four blocks of 128 threads per SM, took 84.5 (FP32) and 59.0
+// (FP16) at 2048^2: its 112 registers left 16 warps to cover the loads.  Three
+// blocks of 2 x 128 threads at 80 registers beat two at 128 (82.3 / 69.8) and four
+// at 64 (spills: 86.7 / 62.4); strips of 64 / 96 / 192 threads 71.9 / 72.7 / 75.5
+// against 71.2 at 128 (FP32).  Separate barriers and one or two more ring rows, so
+// that step 1 may run ahead of step 2, gave nothing (70.0 / 59.1 at five rows, 84.5
+// at six, whose shared memory leaves L1 28 KB).  L2 prefetch of the rows ahead
+// (bulk copies or tensor boxes) was slower at every distance above two rows and on
+// grids that fit L2, and was left out.
 #pragma once
 #include <type_traits>
 
@@ -48,9 +52,9 @@
 
 namespace lbmpf {
 
-// packed arithmetic (F2): FP32 2048^2 71.2 us per step against 72.3 without,
-// walled 2400 x 600 34.1 against 43.1 (before its spills were removed), FP16
-// 58.8 against 59.4
+// packed arithmetic (F2), us per step without -> with: FP32 768^2 12.6 -> 11.8,
+// 2048^2 70.9 -> 69.6, walled 2400 x 600 27.2 -> 26.6; FP16 2048^2 59.5 -> 59.4, 701 x
+// 333 6.7 -> 6.4
 #ifndef LBM_MARCH_PK
 #define LBM_MARCH_PK 1
 #endif
