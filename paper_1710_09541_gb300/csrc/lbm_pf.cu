@@ -1354,9 +1354,11 @@ static lbm_status create_handle(int nx, int ny, const lbm_params* p, void* ws, l
             if (st16 && !h->pm[0].on && bytes * 10.0 < (double)LBM_PREFETCH16_L2X10 * l2) h->pf_ahead = 0;
         }
     }
-    h->tile = plan_tile(nx, ny, *p, sms);
-    h->march = plan_march(nx, ny, *p, sms);
-    if (e == cudaSuccess && h->march.H > 0) {
+    if (e == cudaSuccess) {  // (the plans divide by the number of SMs)
+        h->tile = plan_tile(nx, ny, *p, sms);
+        h->march = plan_march(nx, ny, *p, sms);
+    }
+    if (h->march.H > 0) {
         size_t smem;
         const MarchKernel k = march_kernel(*p, &smem);
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
