@@ -169,7 +169,14 @@ lbm_status lbm_init(lbm_handle* h, const double* phi0, const double* ux0,
  * collision with source F_i (Eqs. 2, 3, 8, 9, 11; d_t(phi u) as the backward
  * difference over one step); the Navier-Stokes collision with forcing G_i
  * (Eqs. 15-17, 20).  Asynchronous on the stream unless check_every triggers
- * a check.  Errors: LBM_ERR_STATE (no init), LBM_ERR_NONFINITE, LBM_ERR_CUDA.
+ * a check.  While the stream is being captured (check_every 0, a stream other
+ * than the default one) the steps are recorded one launch each, and every later
+ * step of the handle takes a launch of its own.  A graph of an even number of
+ * steps can be replayed: it continues from the state that the last replay or a
+ * call with an even number of steps left, and, if it was captured an even number
+ * of steps after an init or restore, from a new init or restore.  The
+ * stochastically rounded format repeats the captured steps' dithers.
+ * Errors: LBM_ERR_STATE (no init), LBM_ERR_NONFINITE, LBM_ERR_CUDA.
  */
 lbm_status lbm_step(lbm_handle* h, int nsteps);
 
@@ -275,6 +282,8 @@ lbm_status lbm_diag_fields_noalloc(const double* d_fields, size_t n, double* d_o
  *   enqueued and marks the batch and every case as failed: the cases answer
  *   LBM_ERR_STATE until lbm_init or lbm_set_state restores them, and the
  *   batch answers LBM_ERR_STATE to every further step (build a new one).
+ *   While the cases' stream is being captured up to 31 steps of a batch
+ *   without checks can be recorded; the rules of lbm_step hold for every case.
  * lbm_batch_info -- for class cls (0: periodic cases, 1: walled cases): the
  *   number of cases, the tile shape in use, its measured microseconds per
  *   step (0 before tuning or for an empty class) and whether tuning ran; any

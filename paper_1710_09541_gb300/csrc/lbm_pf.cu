@@ -662,8 +662,10 @@ __global__ void k_state_in(const float* __restrict__ st, void* __restrict__ fd,
             }
             Pop<ST>::putf(fd, N32, 0, (int)n, c);
         }
-        phiu[n] = st[18 * N + n];
-        phiu[N + n] = st[19 * N + n];
+        if (phiu != st + 18 * N) {  // as in k_state_out
+            phiu[n] = st[18 * N + n];
+            phiu[N + n] = st[19 * N + n];
+        }
     }
 }
 
@@ -784,6 +786,11 @@ struct lbm_handle {
     CUtensorMap pm_phiu1 = {};     // the (phi u) map of phiu[1] (pm's are of phiu[0])
     TileGrid tile = {0, 0, 0};     // tiles of the several-step kernel (S = 0: not used)
     MarchGrid march = {0, 0, 0};   // strips and chunks of the two-step kernel (H = 0: not used)
+    int odd = 0;  // whether an odd number of steps was taken since the last init or restore
+    // a stream capture holds steps of this handle: its steps take one launch each,
+    // and init and restore write buffer `home` (see mark_captured)
+    bool one_step = false;
+    int home = 0;
     char err[512] = {0};
 };
 
@@ -1138,6 +1145,37 @@ static lbm_status launch_march(lbm_handle* h) {
     return LBM_OK;
 }
 
+// Whether stream s is being captured.
+static bool is_capturing(cudaStream_t s) {
+    if (s == nullptr || s == cudaStreamLegacy) return false;  // the legacy stream cannot be
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// A replayed graph works on the buffers that its capture saw, so a captured
+// even number of steps must leave the state in the buffers it started from.
+// One-step launches do: each flips the population buffers and updates (phi u) in
+// place.  Launches of several steps flip both, once for two to six steps.  From
+// the first capture on every step of the handle takes a launch of its own, and
+// init and restore keep to the buffers where an even number of steps now lies, as
+// what happens between the replays must also leave the state where the graph
+// expects it.
+static void mark_captured(lbm_handle* h) {
+    if (h->one_step) return;
+    h->one_step = true;
+    h->home = h->cur ^ h->odd;
+}
+// the buffers that an initial or restored state goes to
+static void first_buffers(lbm_handle* h) {
+    h->cur = h->one_step ? h->home : 0;
+    if (!h->one_step) h->pcur = 0;
+    h->odd = 0;
+}
+
 static lbm_status check_flag(lbm_handle* h) {
     unsigned int v = 0;
     LBM_CUDA(h, cudaMemcpyAsync(&v, h->flag, sizeof v, cudaMemcpyDeviceToHost, h->stream));
@@ -1455,12 +1493,12 @@ lbm_status lbm_init(lbm_handle* h, const double* phi0, const double* ux0, const 
         else
             LBM_CUDA(h, cudaMemsetAsync(in + k * h->N, 0, bytes, h->stream));
     }
-    h->cur = h->pcur = 0;
+    first_buffers(h);
     auto kinit = h->prm.storage == LBM_STORE_FP16_SHIFTED ? k_init<ST_FP16>
                  : is_bf16(h->prm.storage)                ? k_init<ST_BF16>
                                                           : k_init<ST_FP32>;
-    kinit<<<grid1d(h->N), 256, 0, h->stream>>>(in, h->f[0], h->g[0], h->phiu[0], h->nx, h->ny,
-                                                 h->model);
+    kinit<<<grid1d(h->N), 256, 0, h->stream>>>(in, h->f[h->cur], h->g[h->cur], h->phiu[h->pcur], h->nx,
+                                                 h->ny, h->model);
     LBM_CUDA(h, cudaGetLastError());
     LBM_CUDA(h, cudaMemsetAsync(h->flag, 0, sizeof(unsigned int), h->stream));
     LBM_CUDA(h, cudaStreamSynchronize(h->stream));
@@ -1475,15 +1513,17 @@ lbm_status lbm_step(lbm_handle* h, int nsteps) {
     if (nsteps < 0) return fail(h, LBM_ERR_INVALID, "lbm_step: nsteps < 0");
     if (!h->inited) return fail(h, LBM_ERR_STATE, "lbm_step before lbm_init");
     LBM_CUDA(h, cudaSetDevice(h->device));
+    if (!h->one_step && is_capturing(h->stream)) mark_captured(h);
     for (int s = 0; s < nsteps;) {
         // several steps at once, unless a check falls between them
         int n = nsteps - s;
         if (h->prm.check_every > 0 && h->prm.check_every - h->since_check < n)
             n = (int)(h->prm.check_every - h->since_check);
-        n = h->tile.S > 1 ? (n < h->tile.S ? n : h->tile.S) : h->march.H > 0 && n > 1 ? 2 : 1;
+        n = h->one_step ? 1 : h->tile.S > 1 ? (n < h->tile.S ? n : h->tile.S) : h->march.H > 0 && n > 1 ? 2 : 1;
         lbm_status st = n == 1 ? launch_step(h, false) : h->tile.S > 1 ? launch_tile(h, n) : launch_march(h);
         if (st != LBM_OK) return st;
         s += n;
+        h->odd ^= n & 1;
         if (h->prm.check_every > 0 && (h->since_check += n) >= h->prm.check_every) {
             st = check_flag(h);
             if (st != LBM_OK) return st;
@@ -1542,11 +1582,11 @@ lbm_status lbm_set_state(lbm_handle* h, const void* host_buf, size_t bytes) {
     LBM_CUDA(h, cudaSetDevice(h->device));
     float* st = (float*)h->staging;
     LBM_CUDA(h, cudaMemcpyAsync(st, host_buf, bytes, cudaMemcpyHostToDevice, h->stream));
-    h->cur = h->pcur = 0;
+    first_buffers(h);
     auto kin = h->prm.storage == LBM_STORE_FP16_SHIFTED ? k_state_in<ST_FP16>
                : is_bf16(h->prm.storage)                ? k_state_in<ST_BF16>
                                                          : k_state_in<ST_FP32>;
-    kin<<<grid1d(h->N), 256, 0, h->stream>>>(st, h->f[0], h->g[0], h->phiu[0], h->nx,
+    kin<<<grid1d(h->N), 256, 0, h->stream>>>(st, h->f[h->cur], h->g[h->cur], h->phiu[h->pcur], h->nx,
                                                      h->ny, h->model.walls);
     LBM_CUDA(h, cudaGetLastError());
     LBM_CUDA(h, cudaMemsetAsync(h->flag, 0, sizeof(unsigned int), h->stream));
@@ -1982,6 +2022,7 @@ struct lbm_batch {
     bool tuned = false;
     double tuned_us[BATCH_NCLASS][BATCH_NCAND] = {};
     cudaGraphExec_t graph = nullptr;
+    bool graph_pairs = false;  // the graph's launches take two steps each
     bool failed = false;  // a step call failed after enqueueing work (see batch_abort)
     long long node_count = 0;
     char err[512] = {0};
@@ -2066,7 +2107,14 @@ static lbm_status batch_run(lbm_batch* b, long long from, long long to, int pp) 
     return LBM_OK;
 }
 
-static bool batch_marches(const lbm_batch* b) { return b->march[0] + b->march[1] > 0; }
+// whether the batch takes pairs of steps per launch: it has a plan for them, and no
+// stream capture holds steps of a case (mark_captured)
+static bool batch_marches(const lbm_batch* b) {
+    if (b->march[0] + b->march[1] == 0) return false;
+    for (const lbm_handle* h : b->cases)
+        if (h->one_step) return false;
+    return true;
+}
 // n pairs of steps of every non-empty class by the two-step kernel, the first
 // reading the buffers of parities 0
 static lbm_status batch_run_pairs(lbm_batch* b, long long n) {
@@ -2109,8 +2157,9 @@ static lbm_status batch_abort(lbm_batch* b, lbm_status st) {
 }
 
 // after an odd number of launches that changed buffers every case's current ones flip
-static void batch_flip(lbm_batch* b, long long flips, long long pflips) {
+static void batch_flip(lbm_batch* b, long long flips, long long pflips, int nsteps) {
     for (int c = 0; c < b->ncases; ++c) {
+        b->cases[c]->odd ^= nsteps & 1;
         b->cases[c]->cur ^= flips & 1;
         b->cases[c]->pcur ^= pflips & 1;
     }
@@ -2155,10 +2204,11 @@ static lbm_status batch_tune(lbm_batch* b, long long& done) {
 // class a chain of launches on its own stream, the two chains independent.
 static lbm_status batch_capture(lbm_batch* b) {
     cudaGraph_t g;
+    b->graph_pairs = batch_marches(b);
     LBM_BCUDA(b, cudaStreamBeginCapture(b->bs[0], cudaStreamCaptureModeThreadLocal));
     lbm_status st = batch_fork(b);
     if (st == LBM_OK)
-        st = batch_marches(b) ? batch_run_pairs(b, BATCH_GRAPH_STEPS / 2) : batch_run(b, 0, BATCH_GRAPH_STEPS, 0);
+        st = b->graph_pairs ? batch_run_pairs(b, BATCH_GRAPH_STEPS / 2) : batch_run(b, 0, BATCH_GRAPH_STEPS, 0);
     if (st == LBM_OK) st = batch_join(b);
     cudaError_t ce = cudaStreamEndCapture(b->bs[0], &g);
     if (st != LBM_OK) {
@@ -2461,7 +2511,14 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps) {
     // order after earlier work on the cases' stream
     LBM_BCUDA(b, cudaEventRecord(b->ev_in, b->user));
     LBM_BCUDA(b, cudaStreamWaitEvent(b->bs[0], b->ev_in, 0));
+    if (is_capturing(b->user))  // as in lbm_step
+        for (lbm_handle* h : b->cases) mark_captured(h);
+    const bool pairs = batch_marches(b);
     batch_sync_table(b);
+    if (b->graph && b->graph_pairs != pairs) {
+        cudaGraphExecDestroy(b->graph);
+        b->graph = nullptr;
+    }
     lbm_status st;
     if ((st = batch_fork(b)) != LBM_OK) return batch_abort(b, st);
 
@@ -2493,7 +2550,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps) {
     long long flips = done + rest, pflips = 0;
     if (rest > 0) {
         if ((st = batch_fork(b)) != LBM_OK) return batch_abort(b, st);
-        if (batch_marches(b)) {
+        if (pairs) {
             pflips = rest / 2;  // (here `done` is even)
             flips = pflips + (rest & 1);
             if ((st = batch_run_pairs(b, pflips)) != LBM_OK) return batch_abort(b, st);
@@ -2505,7 +2562,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps) {
         if ((st = batch_join(b)) != LBM_OK) return batch_abort(b, st);
     }
     // cases' current buffers (and with them the tables) follow
-    batch_flip(b, flips, pflips);
+    batch_flip(b, flips, pflips, nsteps);
     batch_sync_table(b);
     if (b->check) {
         // the cases' non-finite flags (set by any step of this call), gathered
