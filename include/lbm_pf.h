@@ -181,6 +181,13 @@ lbm_status lbm_init(lbm_handle* h, const double* phi0, const double* ux0,
 lbm_status lbm_step(lbm_handle* h, int nsteps);
 
 /*
+ * lbm_step_launches -- step kernels that lbm_step has launched (or recorded in a
+ * capture) on this handle since it was created; 0 for NULL.  Against the steps
+ * taken it says how many steps a launch takes (LBM_KERNEL_AUTO).
+ */
+long long lbm_step_launches(const lbm_handle* h);
+
+/*
  * lbm_get_fields -- phi, rho, ux, uy, p of the current state, computed by the
  * same formulas as the step (Eqs. 12, 13, 22).  Any output may be NULL.
  * Host arrays of N doubles; synchronises the stream before returning.
@@ -289,12 +296,16 @@ lbm_status lbm_diag_fields_noalloc(const double* d_fields, size_t n, double* d_o
  *   step (0 before tuning or for an empty class) and whether tuning ran; any
  *   output pointer may be NULL.  Errors: LBM_ERR_INVALID (NULL batch, cls not
  *   0 or 1).
+ * lbm_batch_counts -- step kernels launched by lbm_batch_step so far (of both
+ *   classes; a graph replay counts the launches it holds) and CUDA graphs
+ *   captured; either pointer may be NULL.  Errors: LBM_ERR_INVALID (NULL batch).
  */
 typedef struct lbm_batch lbm_batch;
 lbm_status lbm_batch_create(int ncases, lbm_handle* const* cases, lbm_batch** out);
 lbm_status lbm_batch_step(lbm_batch* b, int nsteps);
 lbm_status lbm_batch_info(const lbm_batch* b, int cls, int* ncases, int* tile_tx, int* tile_ty,
                           double* us_per_step, int* tuned);
+lbm_status lbm_batch_counts(const lbm_batch* b, long long* launches, long long* graphs);
 void lbm_batch_destroy(lbm_batch* b);
 const char* lbm_batch_last_error(const lbm_batch* b);
 

@@ -782,6 +782,7 @@ struct lbm_handle {
     int pf_ahead = 0;  // L2 prefetch distance of the step kernel, in tiles
     bool owns_memory = true;  // false: the device buffers live in a caller's workspace
     unsigned long long nstep = 0;  // steps since lbm_init: seeds the stochastic rounding
+    long long launches = 0;        // step kernels launched by lbm_step
     PfMaps pm[2] = {};             // prefetch tensor maps of the step reading buffer 0 / 1
     CUtensorMap pm_phiu1 = {};     // the (phi u) map of phiu[1] (pm's are of phiu[0])
     TileGrid tile = {0, 0, 0};     // tiles of the several-step kernel (S = 0: not used)
@@ -999,7 +1000,10 @@ static lbm_status launch_step(lbm_handle* h, bool fields, const FieldsOut& out =
                                LBM_ALTERNATE_ORDER ? c : 0, pm));
     }
     LBM_CUDA(h, cudaGetLastError());
-    if (!fields) h->cur ^= 1;
+    if (!fields) {
+        h->cur ^= 1;
+        ++h->launches;
+    }
     return LBM_OK;
 }
 
@@ -1125,6 +1129,7 @@ static lbm_status launch_tile(lbm_handle* h, int n) {
     h->nstep += n;
     h->cur ^= 1;
     h->pcur ^= 1;
+    ++h->launches;
     return LBM_OK;
 }
 
@@ -1142,6 +1147,7 @@ static lbm_status launch_march(lbm_handle* h) {
     LBM_CUDA(h, launch_dep(k, grid, dim3(2 * MARCH_TW), smem, h->stream, A, h->model, G, seed2));
     h->cur ^= 1;
     h->pcur ^= 1;
+    ++h->launches;
     return LBM_OK;
 }
 
@@ -1475,6 +1481,8 @@ void lbm_destroy(lbm_handle* h) {
 }
 
 const char* lbm_last_error(const lbm_handle* h) { return h ? h->err : "null handle"; }
+
+long long lbm_step_launches(const lbm_handle* h) { return h ? h->launches : 0; }
 
 size_t lbm_state_bytes(const lbm_handle* h) { return h ? 20 * h->N * sizeof(float) : 0; }
 
@@ -2023,6 +2031,8 @@ struct lbm_batch {
     double tuned_us[BATCH_NCLASS][BATCH_NCAND] = {};
     cudaGraphExec_t graph = nullptr;
     bool graph_pairs = false;  // the graph's launches take two steps each
+    long long launches = 0, graph_launches = 0;  // step kernels launched so far, and those of one replay
+    long long graphs = 0;                        // graphs captured so far
     bool failed = false;  // a step call failed after enqueueing work (see batch_abort)
     long long node_count = 0;
     char err[512] = {0};
@@ -2093,6 +2103,7 @@ static lbm_status batch_launch(lbm_batch* b, int cls, int cand, int parity) {
     LBM_BCUDA(b, launch_dep(k, dim3(b->tiles[cls * BATCH_NCAND + cand]), dim3(BATCH_TX[cand], BATCH_TY[cand]), 0,
                             b->bs[cls], T, (const int2*)b->d_tiles[cls * BATCH_NCAND + cand], parity,
                             b->pf_ahead));
+    ++b->launches;
     return LBM_OK;
 }
 
@@ -2122,9 +2133,11 @@ static lbm_status batch_run_pairs(lbm_batch* b, long long n) {
         if (b->ncls[cls]) {
             size_t smem;
             const MarchBatchKernel k = march_batch_kernel(b->storage, cls, b->check, &smem);
-            for (long long p = 0; p < n; ++p)
+            for (long long p = 0; p < n; ++p) {
                 LBM_BCUDA(b, launch_dep(k, dim3(b->march[cls]), dim3(2 * MARCH_TW), smem, b->bs[cls], b->tab(cls, 0),
                                         (const int4*)b->d_march[cls], (int)(p & 1) * 3));
+                ++b->launches;
+            }
         }
     return LBM_OK;
 }
@@ -2205,12 +2218,15 @@ static lbm_status batch_tune(lbm_batch* b, long long& done) {
 static lbm_status batch_capture(lbm_batch* b) {
     cudaGraph_t g;
     b->graph_pairs = batch_marches(b);
+    const long long before = b->launches;
     LBM_BCUDA(b, cudaStreamBeginCapture(b->bs[0], cudaStreamCaptureModeThreadLocal));
     lbm_status st = batch_fork(b);
     if (st == LBM_OK)
         st = b->graph_pairs ? batch_run_pairs(b, BATCH_GRAPH_STEPS / 2) : batch_run(b, 0, BATCH_GRAPH_STEPS, 0);
     if (st == LBM_OK) st = batch_join(b);
     cudaError_t ce = cudaStreamEndCapture(b->bs[0], &g);
+    b->graph_launches = b->launches - before;
+    b->launches = before;
     if (st != LBM_OK) {
         if (ce == cudaSuccess) cudaGraphDestroy(g);
         return st;
@@ -2222,6 +2238,7 @@ static lbm_status batch_capture(lbm_batch* b) {
         b->graph = nullptr;
         return bfail(b, LBM_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(ce));
     }
+    ++b->graphs;
     return LBM_OK;
 }
 
@@ -2497,6 +2514,13 @@ lbm_status lbm_batch_info(const lbm_batch* b, int cls, int* ncases, int* tile_tx
     return LBM_OK;
 }
 
+lbm_status lbm_batch_counts(const lbm_batch* b, long long* launches, long long* graphs) {
+    if (!b) return LBM_ERR_INVALID;
+    if (launches) *launches = b->launches;
+    if (graphs) *graphs = b->graphs;
+    return LBM_OK;
+}
+
 lbm_status lbm_batch_step(lbm_batch* b, int nsteps) {
     if (!b) return LBM_ERR_INVALID;
     if (b->failed)
@@ -2542,6 +2566,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps) {
             if (ce != cudaSuccess)
                 return batch_abort(b, bfail(b, LBM_ERR_CUDA, "cudaGraphLaunch: %s",
                                             cudaGetErrorString(ce)));
+            b->launches += b->graph_launches;
         }
     }
     // the remainder, with parities continuing from 0 after the replays; flips: the

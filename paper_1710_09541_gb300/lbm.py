@@ -34,7 +34,7 @@ EXPORTS = ("lbm_create", "lbm_init", "lbm_step", "lbm_get_fields", "lbm_state_by
            "lbm_last_error", "lbm_diag_fields_noalloc", "lbm_batch_create", "lbm_batch_step",
            "lbm_batch_info", "lbm_batch_destroy", "lbm_batch_last_error",
            "lbm_spreading_radius", "lbm_probe", "lbm_workspace_bytes", "lbm_create_in",
-           "lbm_laplace_jump")
+           "lbm_laplace_jump", "lbm_step_launches", "lbm_batch_counts")
 
 
 class LbmError(RuntimeError):
@@ -101,6 +101,11 @@ def load() -> ctypes.CDLL:
     L.lbm_batch_info.argtypes = [vp, i, ctypes.POINTER(i), ctypes.POINTER(i), ctypes.POINTER(i), pd,
                                   ctypes.POINTER(i)]
     L.lbm_batch_info.restype = ctypes.c_int
+    L.lbm_step_launches.argtypes = [vp]
+    L.lbm_step_launches.restype = ctypes.c_longlong
+    pll = ctypes.POINTER(ctypes.c_longlong)
+    L.lbm_batch_counts.argtypes = [vp, pll, pll]
+    L.lbm_batch_counts.restype = ctypes.c_int
     L.lbm_batch_destroy.argtypes = [vp]
     L.lbm_batch_destroy.restype = None
     L.lbm_batch_last_error.argtypes = [vp]
@@ -204,6 +209,10 @@ class Lattice:
         self._check(self._L.lbm_step(self._h, int(nsteps)))
         return self
 
+    def step_launches(self) -> int:
+        """Step kernels launched by step() so far (lbm_step_launches)."""
+        return int(self._L.lbm_step_launches(self._h))
+
     def fields(self, out=None):
         """dict phi, rho, ux, uy, p of shape [ny, nx] (float64).  ``out`` may
         supply preallocated (e.g. pinned) arrays for some or all keys."""
@@ -305,6 +314,14 @@ class Batch:
         if rc != LBM_OK:
             raise LbmError(rc, self._L.lbm_batch_last_error(self._h).decode())
         return self
+
+    def counts(self):
+        """(step kernels launched, CUDA graphs captured) so far (lbm_batch_counts)."""
+        n, g = ctypes.c_longlong(), ctypes.c_longlong()
+        rc = self._L.lbm_batch_counts(self._h, ctypes.byref(n), ctypes.byref(g))
+        if rc != LBM_OK:
+            raise LbmError(rc, "lbm_batch_counts failed")
+        return n.value, g.value
 
     def info(self):
         """{"periodic": {...}, "walls": {...}, "tuned": bool}; per class the

@@ -1,0 +1,146 @@
+"""Which kernels the library's rules choose, by the launches they count, and the
+routes that no other test's sizes take.  A comparison of LBM_KERNEL_AUTO with
+LBM_KERNEL_GENERIC says something only where the two take different kernels, so
+each one here first asserts how many steps AUTO took per launch."""
+import numpy as np
+import pytest
+
+from paper_1710_09541_gb300 import cases
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def libs():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1710_09541_gb300 import build as lbm_build
+    from paper_1710_09541_gb300 import lbm
+
+    release, debug = lbm_build.build(), lbm_build.build(debug=True)
+    saved = (lbm._LIB_PATH, lbm._lib)
+    yield lbm, release, debug
+    lbm._LIB_PATH, lbm._lib = saved
+
+
+def _use(lbm, path):
+    lbm._LIB_PATH, lbm._lib = path, None
+
+
+def _same(a, b):
+    assert np.isfinite(a[0]).all()
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
+
+
+def _run(lbm, nx, ny, bc, storage, steps, kernel):
+    P = dict(rho_l=1.0, rho_g=0.01, nu_l=0.05, nu_g=0.1, visc_mode=0, sigma=1e-3, W=4.0, tau_h=0.8,
+             Gx=1e-6, Gy=-2e-6, bc_y=bc)
+    with lbm.Lattice(nx, ny, storage=storage, kernel=kernel, **P) as g:
+        g.init(cases.spinodal(nx, ny, 0.5, 0.2, seed=nx + ny), 1e-3 * cases.spinodal(nx, ny, 0.0, 1.0, seed=7))
+        g.step(steps)
+        return g.step_launches(), [*g.get_state(), *g.fields().values()]
+
+
+# one narrow strip; a low and wide grid; rows of whole sectors in every format
+MARCHING = [(65, 9000, 0), (67, 20000, 1), (67, 20000, 2), (67, 20000, 3), (20001, 16, 0), (20001, 16, 1),
+            (1280, 1280, 0), (1280, 1280, 1), (1280, 1280, 2), (1280, 1280, 3), (701, 333, 0), (123, 4700, 0)]
+
+
+@pytest.mark.parametrize("nx,ny,storage", MARCHING)
+@pytest.mark.parametrize("bc", [0, 1, 2])
+def test_march_where_it_is_chosen(libs, nx, ny, storage, bc):
+    lbm, release, _ = libs
+    _use(lbm, release)
+    n, got = _run(lbm, nx, ny, bc, storage, 9, 0)
+    assert n == 5  # four pairs and one step
+    m, want = _run(lbm, nx, ny, bc, storage, 9, 1)
+    assert m == 9
+    _same(got, want)
+
+
+@pytest.mark.parametrize("nx,ny,storage,per_launch", [(64, 64, 0, 3), (8, 256, 0, 3), (200, 200, 2, 2), (3, 5, 1, 4),
+                                                      (1, 64, 0, 1), (512, 512, 0, 1), (1024, 1024, 1, 1)])
+def test_steps_per_launch(libs, nx, ny, storage, per_launch):
+    lbm, release, _ = libs
+    _use(lbm, release)
+    n, got = _run(lbm, nx, ny, 0, storage, 12, 0)
+    assert n == 12 // per_launch
+    if per_launch > 1:
+        _same(got, _run(lbm, nx, ny, 0, storage, 12, 1)[1])
+
+
+# 8.7 M nodes in strips close to 122 columns, so that 16-bit batches march; both classes
+LARGE = [(976, 960, 0), (976, 960, 1), (1098, 801, 0), (1220, 640, 2), (973, 1100, 0), (976, 720, 1), (610, 1300, 0),
+         (1097, 900, 1), (976, 960, 2), (366, 1500, 0)]
+
+
+def _batch(lbm, specs, storage, kernel, steps, check_every=0):
+    lats = []
+    for nx, ny, bc in specs:
+        P = dict(cases.params_spinodal(), bc_y=bc, check_every=check_every)
+        lats.append(lbm.Lattice(nx, ny, storage=storage, kernel=kernel, **P).init(cases.spinodal(nx, ny, seed=nx + ny)))
+    try:
+        with lbm.Batch(lats) as bt:
+            counts = []
+            for k in steps:
+                bt.step(k)
+                counts.append(bt.counts()[0])
+                lats[2].step(3)  # a case stepped on its own in between
+        return counts, [a for lat in lats for a in lat.get_state()]
+    finally:
+        for lat in lats:
+            lat.close()
+
+
+@pytest.mark.parametrize("storage,check_every", [(1, 0), (2, 0), (1, 2), (2, 1)])
+def test_16bit_batch_march(libs, storage, check_every):
+    """Fewer steps than a graph, odd counts, graph replays with even and odd
+    remainders; with checks also through the index-checking build."""
+    lbm, release, debug = libs
+    steps = (7, 4, 1, 67, 34)
+    _use(lbm, release)
+    n, got = _batch(lbm, LARGE, storage, 0, steps, check_every)
+    assert n == [8, 12, 14, 82, 116]  # per class: 3 + 1, 2, 1, 32 + 1 + 1, 16 + 1
+    m, want = _batch(lbm, LARGE, storage, 1, steps, check_every)
+    assert m[-1] == 2 * sum(steps)
+    _same(got, want)
+    if check_every:
+        _use(lbm, debug)
+        n, again = _batch(lbm, LARGE, storage, 0, steps, check_every)
+        assert n[-1] == 116
+        _same(again, want)
+
+
+@pytest.mark.parametrize("odd", [False, True])
+def test_prefetching_batch_steps(libs, odd):
+    """One-step launches of a 16-bit batch above the prefetch threshold (tensor
+    maps; with one more case of nx = 1004 per-thread requests) against cases
+    stepped alone: the two-step launches leave this path only to GENERIC cases
+    and to batches below their own threshold."""
+    lbm, release, _ = libs
+    _use(lbm, release)
+    specs = cases.batch_cases(24, seed=11)  # 6 M nodes: 552 MB a step
+    if odd:
+        phi0 = cases.drop(1004, 300, 40.0, 4.0)
+        specs.append(dict(nx=1004, ny=300, params=cases.params_static_drop(ratio=100.0), phi0=phi0, ux0=None, uy0=None))
+    pick = [0, 1, 23, len(specs) - 1]
+
+    def make(which, kernel):
+        return [lbm.Lattice(sp["nx"], sp["ny"], storage=1, kernel=kernel, **sp["params"])
+                .init(sp["phi0"], sp["ux0"], sp["uy0"]) for sp in which]
+
+    A, B = make(specs, 1), make([specs[k] for k in pick], 1)
+    try:
+        with lbm.Batch(A) as bt:
+            bt.step(10)
+            assert bt.counts()[0] == 20
+        for lat in B:
+            lat.step(10)
+        for k, b in zip(pick, B):
+            _same(A[k].get_state(), b.get_state())
+    finally:
+        for lat in A + B:
+            lat.close()
