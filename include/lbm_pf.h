@@ -277,7 +277,9 @@ lbm_status lbm_diag_fields_noalloc(const double* d_fields, size_t n, double* d_o
  *   run concurrently.  Steps run as replays of a CUDA graph of 32 steps per class.  The first call with
  *   nsteps >= 140 times five tile shapes (32x4, 32x8, 32x16, 64x2, 64x4 nodes)
  *   for each class on its own first 140 steps (per shape 4 warm-up steps and
- *   the faster of two windows of 12) and keeps the fastest.
+ *   the faster of two windows of 12) and keeps the fastest.  A batch that takes
+ *   pairs of steps per launch has no shape to choose: that call times 12 of its
+ *   own steps per class, and a call's odd step takes the 32x8 shape.
  *   Ordered after earlier work on the cases' stream, and later work on that
  *   stream waits for it.  A case may also be stepped on its own between batch
  *   steps.  If any case was created with check_every > 0, the call ends by
@@ -292,9 +294,11 @@ lbm_status lbm_diag_fields_noalloc(const double* d_fields, size_t n, double* d_o
  *   While the cases' stream is being captured up to 31 steps of a batch
  *   without checks can be recorded; the rules of lbm_step hold for every case.
  * lbm_batch_info -- for class cls (0: periodic cases, 1: walled cases): the
- *   number of cases, the tile shape in use, its measured microseconds per
- *   step (0 before tuning or for an empty class) and whether tuning ran; any
- *   output pointer may be NULL.  Errors: LBM_ERR_INVALID (NULL batch, cls not
+ *   number of cases, the tile shape in use for single steps, the measured
+ *   microseconds per step (0 before tuning or for an empty class) and whether
+ *   tuning ran.  In a batch that takes pairs of steps per launch the time is that
+ *   of the pairs, whose launches have no tile shape; otherwise it is the tile
+ *   shape's.  Any output pointer may be NULL.  Errors: LBM_ERR_INVALID (NULL batch, cls not
  *   0 or 1).
  * lbm_batch_counts -- step kernels launched by lbm_batch_step so far (of both
  *   classes; a graph replay counts the launches it holds) and CUDA graphs

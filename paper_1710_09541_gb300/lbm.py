@@ -325,8 +325,9 @@ class Batch:
 
     def info(self):
         """{"periodic": {...}, "walls": {...}, "tuned": bool}; per class the
-        number of cases, the tile shape (width, height) in use and its
-        microseconds per step at tuning."""
+        number of cases, the tile shape (width, height) in use for single steps
+        and the measured microseconds per step, of that shape or, where the
+        batch takes pairs of steps per launch, of the pairs (lbm_batch_info)."""
         out = {}
         for cls, name in ((0, "periodic"), (1, "walls")):
             n, tx, ty, tuned = ctypes.c_int(), ctypes.c_int(), ctypes.c_int(), ctypes.c_int()

@@ -144,3 +144,28 @@ def test_prefetching_batch_steps(libs, odd):
     finally:
         for lat in A + B:
             lat.close()
+
+
+@pytest.mark.parametrize("storage,pairs", [(0, True), (1, False)])
+def test_first_long_batch_call(libs, storage, pairs):
+    """The first call of 140 or more steps times what the batch runs: pairs of
+    steps (no one-step launch then), or the tile shapes."""
+    lbm, release, _ = libs
+    _use(lbm, release)
+    specs = cases.batch_cases(16, seed=11)
+    lats = [lbm.Lattice(sp["nx"], sp["ny"], storage=storage, **sp["params"]).init(sp["phi0"], sp["ux0"], sp["uy0"])
+            for sp in specs]
+    alone = [lbm.Lattice(sp["nx"], sp["ny"], storage=storage, kernel=lbm.LBM_KERNEL_GENERIC, **sp["params"])
+             .init(sp["phi0"], sp["ux0"], sp["uy0"]).step(161) for sp in specs[:3]]
+    try:
+        with lbm.Batch(lats) as bt:
+            assert not bt.info()["tuned"]
+            bt.step(161)
+            assert bt.counts()[0] == 2 * (81 if pairs else 161)
+            info = bt.info()
+            assert info["tuned"] and info["periodic"]["us"] > 0 and info["walls"]["us"] > 0
+        for a, b in zip(lats, alone):
+            _same(a.get_state(), b.get_state())
+    finally:
+        for lat in lats + alone:
+            lat.close()
