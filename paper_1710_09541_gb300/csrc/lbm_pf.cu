@@ -1804,7 +1804,7 @@ struct CaseDesc {
     float* phiu[2];
     unsigned int* flag;
     int nx, ny;
-    int cur;   // buffers holding the current state when the batch parities are 0 (bits as parity's)
+    int cur;   // buffers holding the current state when the launch's parity is 0 (bits as parity's)
     int map0;  // first of the case's 8 prefetch maps in BatchTable::maps (4 per buffer)
     Model m;
 };
@@ -2032,10 +2032,14 @@ struct lbm_batch {
     double tuned_us[BATCH_NCLASS][BATCH_NCAND] = {};
     bool pairs_timed = false;  // the two-step kernel's time per step, for lbm_batch_info
     double pairs_us[BATCH_NCLASS] = {};
-    cudaGraphExec_t graph = nullptr;
-    bool graph_pairs = false;  // the graph's launches take two steps each
-    long long launches = 0, graph_launches = 0;  // step kernels launched so far, and those of one replay
-    long long graphs = 0;                        // graphs captured so far
+    // the buffers of the current state against the tables' (bits as parity's), the
+    // same for every case
+    int off = 0;
+    // captured steps, one per launch or in pairs ([1]), by the parity of the first launch
+    cudaGraphExec_t graph[2][4] = {};
+    bool stale = false;  // they hold other tables (none may be destroyed while a stream is captured)
+    long long graph_launches[2] = {0, 0};  // step kernels of one replay
+    long long launches = 0, graphs = 0;    // step kernels launched and graphs captured so far
     bool failed = false;  // a step call failed after enqueueing work (see batch_abort)
     long long node_count = 0;
     char err[512] = {0};
@@ -2060,8 +2064,17 @@ static lbm_status bfail(lbm_batch* b, lbm_status st, const char* fmt, ...) {
                          __FILE__, __LINE__);                                               \
     } while (0)
 
+static void batch_drop_graphs(lbm_batch* b) {
+    for (auto& kind : b->graph)
+        for (cudaGraphExec_t& g : kind) {
+            if (g) cudaGraphExecDestroy(g);
+            g = nullptr;
+        }
+    b->stale = false;
+}
+
 static void batch_release(lbm_batch* b) {
-    if (b->graph) cudaGraphExecDestroy(b->graph);
+    batch_drop_graphs(b);
     delete[] b->table;
     for (int2* t : b->d_tiles)
         if (t) cudaFree(t);
@@ -2077,24 +2090,24 @@ static void batch_release(lbm_batch* b) {
         if (b->bs[k]) cudaStreamDestroy(b->bs[k]);
 }
 
-// Take each case's current buffer from its handle (a case may have been
-// stepped on its own since the last batch step); a change invalidates the
-// captured graph, whose launches carry the tables.
+// Take each case's current buffers from its handle (a case may have been stepped
+// on its own since the last batch step).  Cases that all moved alike are an
+// offset of the parity; only otherwise do the tables change, and with them the
+// captured graphs, whose launches carry them.  (With every move in the tables, each
+// call whose launches changed buffers an odd number of times captured a new
+// graph: 16 cases with FP32 storage took 84.5 us per step in calls of 50 steps,
+// 84.1 in calls of 52.)
 static void batch_sync_table(lbm_batch* b) {
-    bool changed = false;
+    auto now = [&](int c) { return b->cases[c]->cur | b->cases[c]->pcur << 1; };
+    auto desc = [&](int c, int k) -> CaseDesc& { return b->tab(b->cls_of[c], k).c[b->slot_of[c]]; };
+    const int off = now(0) ^ desc(0, 0).cur;
+    bool alike = true;
+    for (int c = 1; c < b->ncases; ++c) alike = alike && (now(c) ^ desc(c, 0).cur) == off;
+    b->off = alike ? off : 0;
+    if (alike) return;
     for (int c = 0; c < b->ncases; ++c)
-        for (int k = 0; k < BATCH_NCAND; ++k) {
-            CaseDesc& d = b->tab(b->cls_of[c], k).c[b->slot_of[c]];
-            const int now = b->cases[c]->cur | b->cases[c]->pcur << 1;
-            if (d.cur != now) {
-                d.cur = now;
-                changed = true;
-            }
-        }
-    if (changed && b->graph) {
-        cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
-    }
+        for (int k = 0; k < BATCH_NCAND; ++k) desc(c, k).cur = now(c);
+    b->stale = true;
 }
 
 // one step of class cls with tile shape cand, on the class's stream
@@ -2110,14 +2123,14 @@ static lbm_status batch_launch(lbm_batch* b, int cls, int cand, int parity) {
     return LBM_OK;
 }
 
-// steps [from, to) of every non-empty class, each class on its own stream, with
-// (phi u) in the buffers of parity pp
-static lbm_status batch_run(lbm_batch* b, long long from, long long to, int pp) {
+// n steps of every non-empty class, one per launch, each class on its own
+// stream; parity: of the first launch
+static lbm_status batch_run(lbm_batch* b, long long n, int parity) {
     lbm_status st;
     for (int cls = 0; cls < BATCH_NCLASS; ++cls)
         if (b->ncls[cls])
-            for (long long s = from; s < to; ++s)
-                if ((st = batch_launch(b, cls, b->cand[cls], (int)(s & 1) | pp << 1)) != LBM_OK) return st;
+            for (long long s = 0; s < n; ++s)
+                if ((st = batch_launch(b, cls, b->cand[cls], parity ^ (int)(s & 1))) != LBM_OK) return st;
     return LBM_OK;
 }
 
@@ -2129,23 +2142,22 @@ static bool batch_marches(const lbm_batch* b) {
         if (h->one_step) return false;
     return true;
 }
-// n pairs of steps of class cls by the two-step kernel, the first reading the
-// buffers of parities 0
-static lbm_status batch_run_pairs(lbm_batch* b, int cls, long long n) {
+// n pairs of steps of class cls by the two-step kernel; parity: of the first launch
+static lbm_status batch_run_pairs(lbm_batch* b, int cls, long long n, int parity) {
     size_t smem;
     const MarchBatchKernel k = march_batch_kernel(b->storage, cls, b->check, &smem);
     for (long long p = 0; p < n; ++p) {
         LBM_BCUDA(b, launch_dep(k, dim3(b->march[cls]), dim3(2 * MARCH_TW), smem, b->bs[cls], b->tab(cls, 0),
-                                (const int4*)b->d_march[cls], (int)(p & 1) * 3));
+                                (const int4*)b->d_march[cls], parity ^ (int)(p & 1) * 3));
         ++b->launches;
     }
     return LBM_OK;
 }
 // the same of every non-empty class
-static lbm_status batch_run_pairs(lbm_batch* b, long long n) {
+static lbm_status batch_run_pairs(lbm_batch* b, long long n, int parity) {
     lbm_status st;
     for (int cls = 0; cls < BATCH_NCLASS; ++cls)
-        if (b->ncls[cls] && (st = batch_run_pairs(b, cls, n)) != LBM_OK) return st;
+        if (b->ncls[cls] && (st = batch_run_pairs(b, cls, n, parity)) != LBM_OK) return st;
     return LBM_OK;
 }
 
@@ -2176,13 +2188,15 @@ static lbm_status batch_abort(lbm_batch* b, lbm_status st) {
     return st;
 }
 
-// after an odd number of launches that changed buffers every case's current ones flip
-static void batch_flip(lbm_batch* b, long long flips, long long pflips, int nsteps) {
-    for (int c = 0; c < b->ncases; ++c) {
-        b->cases[c]->odd ^= nsteps & 1;
-        b->cases[c]->cur ^= flips & 1;
-        b->cases[c]->pcur ^= pflips & 1;
+// the cases' current buffers after nsteps steps that left the launches' parity at `parity`
+static void batch_set_off(lbm_batch* b, int parity, int nsteps) {
+    const int flip = parity ^ b->off;
+    for (lbm_handle* h : b->cases) {
+        h->odd ^= nsteps & 1;
+        h->cur ^= flip & 1;
+        h->pcur ^= flip >> 1;
     }
+    b->off = parity;
 }
 
 // Time every tile shape of each class on the live state (all shapes give the
@@ -2196,12 +2210,12 @@ static lbm_status batch_tune(lbm_batch* b, long long& done) {
         double best = 1e300;
         for (int k = 0; k < BATCH_NCAND; ++k) {
             for (int w = 0; w < BATCH_TUNE_WARM; ++w, ++s)
-                if ((st = batch_launch(b, cls, k, (int)(s & 1))) != LBM_OK) return st;
+                if ((st = batch_launch(b, cls, k, b->off ^ (int)(s & 1))) != LBM_OK) return st;
             double us = 1e300;
             for (int win = 0; win < BATCH_TUNE_WINDOWS; ++win) {
                 LBM_BCUDA(b, cudaEventRecord(b->t0, b->bs[cls]));
                 for (int w = 0; w < BATCH_TUNE_WINDOW; ++w, ++s)
-                    if ((st = batch_launch(b, cls, k, (int)(s & 1))) != LBM_OK) return st;
+                    if ((st = batch_launch(b, cls, k, b->off ^ (int)(s & 1))) != LBM_OK) return st;
                 LBM_BCUDA(b, cudaEventRecord(b->t1, b->bs[cls]));
                 LBM_BCUDA(b, cudaEventSynchronize(b->t1));
                 float ms = 0.f;
@@ -2224,16 +2238,16 @@ static lbm_status batch_tune(lbm_batch* b, long long& done) {
 // other, where it takes the batch's pairs of steps.  There is nothing to choose,
 // so this takes 16 steps; the tile shapes, which such a batch uses for a call's odd
 // step only, are not timed (140 one-step launches per class cost a first call of
-// 160 steps 17.9 ms instead of 14.0, 16 cases with FP32 storage).
+// 160 steps 17.9 ms instead of 14.3, 16 cases with FP32 storage).
 static lbm_status batch_time_pairs(lbm_batch* b, long long& done) {
     constexpr int warm = BATCH_TUNE_WARM / 2, pairs = BATCH_TUNE_WINDOW / 2;
-    static_assert((warm + pairs) % 2 == 0, "the parities return to 0");
+    static_assert(warm % 2 == 0 && pairs % 2 == 0, "the parity returns to its start");
     lbm_status st;
     for (int cls = 0; cls < BATCH_NCLASS; ++cls) {
         if (!b->ncls[cls]) continue;
-        if ((st = batch_run_pairs(b, cls, warm)) != LBM_OK) return st;
+        if ((st = batch_run_pairs(b, cls, warm, b->off)) != LBM_OK) return st;
         LBM_BCUDA(b, cudaEventRecord(b->t0, b->bs[cls]));
-        if ((st = batch_run_pairs(b, cls, pairs)) != LBM_OK) return st;
+        if ((st = batch_run_pairs(b, cls, pairs, b->off)) != LBM_OK) return st;
         LBM_BCUDA(b, cudaEventRecord(b->t1, b->bs[cls]));
         LBM_BCUDA(b, cudaEventSynchronize(b->t1));
         float ms = 0.f;
@@ -2245,29 +2259,29 @@ static lbm_status batch_time_pairs(lbm_batch* b, long long& done) {
     return LBM_OK;
 }
 
-// Capture BATCH_GRAPH_STEPS steps (parities 0, 1, ..., or as many in pairs) of both classes, each
-// class a chain of launches on its own stream, the two chains independent.
-static lbm_status batch_capture(lbm_batch* b) {
+// Capture BATCH_GRAPH_STEPS steps of both classes from the
+// launch parity `parity`, each class a chain of launches on its own stream, the
+// two chains independent; pairs: two steps per launch.
+static lbm_status batch_capture(lbm_batch* b, bool pairs, int parity) {
     cudaGraph_t g;
-    b->graph_pairs = batch_marches(b);
     const long long before = b->launches;
     LBM_BCUDA(b, cudaStreamBeginCapture(b->bs[0], cudaStreamCaptureModeThreadLocal));
     lbm_status st = batch_fork(b);
     if (st == LBM_OK)
-        st = b->graph_pairs ? batch_run_pairs(b, BATCH_GRAPH_STEPS / 2) : batch_run(b, 0, BATCH_GRAPH_STEPS, 0);
+        st = pairs ? batch_run_pairs(b, BATCH_GRAPH_STEPS / 2, parity) : batch_run(b, BATCH_GRAPH_STEPS, parity);
     if (st == LBM_OK) st = batch_join(b);
     cudaError_t ce = cudaStreamEndCapture(b->bs[0], &g);
-    b->graph_launches = b->launches - before;
+    b->graph_launches[pairs] = b->launches - before;
     b->launches = before;
     if (st != LBM_OK) {
         if (ce == cudaSuccess) cudaGraphDestroy(g);
         return st;
     }
     if (ce != cudaSuccess) return bfail(b, LBM_ERR_CUDA, "graph capture: %s", cudaGetErrorString(ce));
-    ce = cudaGraphInstantiate(&b->graph, g, 0);
+    ce = cudaGraphInstantiate(&b->graph[pairs][parity], g, 0);
     cudaGraphDestroy(g);
     if (ce != cudaSuccess) {
-        b->graph = nullptr;
+        b->graph[pairs][parity] = nullptr;
         return bfail(b, LBM_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(ce));
     }
     ++b->graphs;
@@ -2568,14 +2582,12 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps) {
     // order after earlier work on the cases' stream
     LBM_BCUDA(b, cudaEventRecord(b->ev_in, b->user));
     LBM_BCUDA(b, cudaStreamWaitEvent(b->bs[0], b->ev_in, 0));
-    if (is_capturing(b->user))  // as in lbm_step
+    const bool capturing = is_capturing(b->user);
+    if (capturing)  // as in lbm_step
         for (lbm_handle* h : b->cases) mark_captured(h);
     const bool pairs = batch_marches(b);
     batch_sync_table(b);
-    if (b->graph && b->graph_pairs != pairs) {
-        cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
-    }
+    if (b->stale && !capturing) batch_drop_graphs(b);
     lbm_status st;
     if ((st = batch_fork(b)) != LBM_OK) return batch_abort(b, st);
 
@@ -2586,44 +2598,34 @@ lbm_status lbm_batch_step(lbm_batch* b, int nsteps) {
         if (pairs && !b->pairs_timed && (st = batch_time_pairs(b, done)) != LBM_OK) return batch_abort(b, st);
         if (!pairs && !b->tuned && (st = batch_tune(b, done)) != LBM_OK) return batch_abort(b, st);
     }
-    // an odd count so far: one more step so the graph starts at parity 0
-    if ((done & 1) && done < nsteps) {
-        if ((st = batch_run(b, done, done + 1, 0)) != LBM_OK) return batch_abort(b, st);
-        ++done;
-    }
     if ((st = batch_join(b)) != LBM_OK) return batch_abort(b, st);
-    // whole graph replays (BATCH_GRAPH_STEPS steps each, parity returns to 0)
+    // whole graph replays (an even number of launches each, as so far: the parity
+    // is still the first one)
+    int parity = b->off;
     const long long reps = (nsteps - done) / BATCH_GRAPH_STEPS;
     if (reps > 0) {
-        if (!b->graph && (st = batch_capture(b)) != LBM_OK) return batch_abort(b, st);
+        cudaGraphExec_t& graph = b->graph[pairs][parity];
+        if (!graph && (st = batch_capture(b, pairs, parity)) != LBM_OK) return batch_abort(b, st);
         for (long long r = 0; r < reps; ++r) {
-            const cudaError_t ce = cudaGraphLaunch(b->graph, b->bs[0]);
+            const cudaError_t ce = cudaGraphLaunch(graph, b->bs[0]);
             if (ce != cudaSuccess)
                 return batch_abort(b, bfail(b, LBM_ERR_CUDA, "cudaGraphLaunch: %s",
                                             cudaGetErrorString(ce)));
-            b->launches += b->graph_launches;
+            b->launches += b->graph_launches[pairs];
         }
     }
-    // the remainder, with parities continuing from 0 after the replays; flips: the
-    // launches that changed buffers since the parity was 0
-    const long long at = done + reps * BATCH_GRAPH_STEPS, rest = nsteps - at;
-    long long flips = done + rest, pflips = 0;
+    // the remainder: pairs, then single steps
+    const long long rest = nsteps - done - reps * BATCH_GRAPH_STEPS;
     if (rest > 0) {
+        const long long np = pairs ? rest / 2 : 0, singles = rest - 2 * np;
         if ((st = batch_fork(b)) != LBM_OK) return batch_abort(b, st);
-        if (pairs) {
-            pflips = rest / 2;  // (here `done` is even)
-            flips = pflips + (rest & 1);
-            if ((st = batch_run_pairs(b, pflips)) != LBM_OK) return batch_abort(b, st);
-            if ((rest & 1) && (st = batch_run(b, pflips, pflips + 1, (int)(pflips & 1))) != LBM_OK)
-                return batch_abort(b, st);
-        } else if ((st = batch_run(b, at, nsteps, 0)) != LBM_OK) {
-            return batch_abort(b, st);
-        }
+        if ((st = batch_run_pairs(b, np, parity)) != LBM_OK) return batch_abort(b, st);
+        parity ^= (int)(np & 1) * 3;
+        if ((st = batch_run(b, singles, parity)) != LBM_OK) return batch_abort(b, st);
+        parity ^= (int)(singles & 1);
         if ((st = batch_join(b)) != LBM_OK) return batch_abort(b, st);
     }
-    // cases' current buffers (and with them the tables) follow
-    batch_flip(b, flips, pflips, nsteps);
-    batch_sync_table(b);
+    batch_set_off(b, parity, nsteps);
     if (b->check) {
         // the cases' non-finite flags (set by any step of this call), gathered
         // and cleared on the device, then read on the host

@@ -99,12 +99,16 @@ def test_captured_batch_steps_replay(env, before):
     try:
         with lbm.Batch(A) as bt, lbm.Batch(B) as ref:
             bt.step(before)
+            for lat in A[:8]:           # moves some cases' buffers
+                lat.step(2)
             g = _capture(torch, s, lambda: bt.step(6))
             _replay(torch, s, g, 3)
             bt.step(34)
             A[2].step(4)
             _replay(torch, s, g, 1)
             ref.step(before + 18 + 34)
+            for lat in B[:8]:
+                lat.step(2)
             B[2].step(4)
             ref.step(6)
             for a, b in zip(A, B):

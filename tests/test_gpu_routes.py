@@ -169,3 +169,40 @@ def test_first_long_batch_call(libs, storage, pairs):
     finally:
         for lat in lats + alone:
             lat.close()
+
+
+@pytest.mark.parametrize("storage,n", [(0, 50), (0, 47), (1, 33)])
+def test_batch_graphs_are_kept(libs, storage, n):
+    """Calls that leave the state in other buffers than they found it in (50: an
+    odd number of pairs, 47: of pairs and a step, 33: of single steps) replay one
+    graph per starting buffer; a case stepped on its own makes new ones."""
+    lbm, release, _ = libs
+    _use(lbm, release)
+    specs = cases.batch_cases(8, seed=11)
+
+    def make(kernel):
+        return [lbm.Lattice(sp["nx"], sp["ny"], storage=storage, kernel=kernel, **sp["params"])
+                .init(sp["phi0"], sp["ux0"], sp["uy0"]) for sp in specs]
+
+    A, B = make(0), make(1)
+    try:
+        with lbm.Batch(A) as bt:
+            for _ in range(8):
+                bt.step(n)
+            assert bt.counts()[1] == {50: 2, 47: 2, 33: 2}[n]
+            for lat in B:
+                lat.step(8 * n)
+            for a, b in zip(A, B):
+                _same(a.get_state(), b.get_state())
+            A[3].step(1)
+            B[3].step(1)
+            for _ in range(5):
+                bt.step(n)
+            assert bt.counts()[1] == 4
+            for lat in B:
+                lat.step(5 * n)
+            for a, b in zip(A, B):
+                _same((*a.get_state(), *a.fields().values()), (*b.get_state(), *b.fields().values()))
+    finally:
+        for lat in A + B:
+            lat.close()
