@@ -1805,7 +1805,7 @@ struct CaseDesc {
     unsigned int* flag;
     int nx, ny;
     int cur;   // buffers holding the current state when the launch's parity is 0 (bits as parity's)
-    int map0;  // first of the case's 8 prefetch maps in BatchTable::maps (4 per buffer)
+    int map0;  // first of the case's 8 prefetch maps in BatchTable::maps: 4 per buffer, the last its (phi u)
     Model m;
 };
 
@@ -1816,6 +1816,9 @@ constexpr int BATCH_MAX_CASES = 200;
 constexpr int BATCH_PF_BOX_X = 32, BATCH_PF_BOX_Y = 10;
 struct BatchTable {
     const CUtensorMap* maps;  // 16-bit prefetch maps in device memory (nullptr: per-thread requests)
+#if LBM_DEBUG_CHECKS
+    const void* const* bases;  // the address that each of them starts at
+#endif
     int ncases;
     CaseDesc c[BATCH_MAX_CASES];
 };
@@ -1865,7 +1868,7 @@ __global__ void __launch_bounds__(TX* TY, (ST == ST_FP32 ? LBM_BATCH_THREADS : L
     if (pf_ahead > 0 && blockIdx.x + pf_ahead < gridDim.x) {
         const int2 pe = __ldg(tiles + (rev ? slot - pf_ahead : slot + pf_ahead));
         const CaseDesc& pc = T.c[pe.x < T.ncases ? pe.x : 0];
-        const int pcur = (pc.cur + parity) & 1;
+        const int pcur = (pc.cur + parity) & 1, ppu = ((pc.cur >> 1) + (parity >> 1)) & 1;
         if (ST != ST_FP32 && T.maps != nullptr) {
             // through the case's tensor maps, boxes of 32 x 10 elements:
             // (TX / 32) x ceil((TH + 2) / 10) boxes per map, one box of one
@@ -1878,14 +1881,22 @@ __global__ void __launch_bounds__(TX* TY, (ST == ST_FP32 ? LBM_BATCH_THREADS : L
                 const int x = (pe.y & 0xffff) * TX + BATCH_PF_BOX_X * (sub % SX);
                 const int r0 = (pe.y >> 16) * TH;
                 const int y = (r0 > 0 ? r0 - 1 : 0) + BATCH_PF_BOX_Y * (sub / SX);
-                const CUtensorMap* mp = T.maps + pc.map0 + 4 * pcur + k;
+                const int mi = pc.map0 + 4 * (k == 3 ? ppu : pcur) + k;
+                const CUtensorMap* mp = T.maps + mi;
+#if LBM_DEBUG_CHECKS
+                const char* const want = k == 0   ? (const char*)pc.f[pcur] + (size_t)4 * pc.nx * pc.ny
+                                         : k == 1 ? (const char*)pc.f[pcur]
+                                         : k == 2 ? (const char*)pc.g[pcur]
+                                                  : (const char*)pc.phiu[ppu];
+                if (T.bases[mi] != want) atomicOr(pc.flag, 4u);
+#endif
                 if (k == 1 || k == 2)
                     tma_prefetch_2d(mp, x, y);
                 else
                     tma_prefetch_3d(mp, x, y, 0);
             }
         } else {
-            prefetch_tile<TX, TH, TX * TY, ST>(pc.f[pcur], pc.g[pcur], pc.phiu[((pc.cur >> 1) + (parity >> 1)) & 1], pc.nx, pc.ny, WALLS,
+            prefetch_tile<TX, TH, TX * TY, ST>(pc.f[pcur], pc.g[pcur], pc.phiu[ppu], pc.nx, pc.ny, WALLS,
                                                pe.y & 0xffff, pe.y >> 16);
         }
     }
@@ -2026,6 +2037,9 @@ struct lbm_batch {
     int cand[BATCH_NCLASS] = {1, 1};  // tile shape in use per class (index into BATCH_TX/TY)
     int pf_ahead = 0;                 // L2 prefetch distance in tiles (0: off)
     CUtensorMap* d_maps = nullptr;    // the 16-bit prefetch maps, 8 per case (nullptr: none)
+#if LBM_DEBUG_CHECKS
+    const void** d_bases = nullptr;
+#endif
     int4* d_march[BATCH_NCLASS] = {};  // the two-step kernel's block lists, and their lengths
     int march[BATCH_NCLASS] = {0, 0};  // (0 in both: not used)
     bool tuned = false;
@@ -2082,6 +2096,9 @@ static void batch_release(lbm_batch* b) {
         if (t) cudaFree(t);
     if (b->d_flags) cudaFree(b->d_flags);
     if (b->d_maps) cudaFree(b->d_maps);
+#if LBM_DEBUG_CHECKS
+    if (b->d_bases) cudaFree(b->d_bases);
+#endif
     for (int4* t : b->d_march)
         if (t) cudaFree(t);
     for (cudaEvent_t e : {b->ev_in, b->ev_out, b->ev_fork, b->ev_join, b->t0, b->t1})
@@ -2497,8 +2514,20 @@ lbm_status lbm_batch_create(int ncases, lbm_handle* const* cases, lbm_batch** ou
                 std::vector<CUtensorMap> maps((size_t)ncases * 8);
                 bool ok = true;
                 for (int c = 0; c < ncases && ok; ++c)
-                    ok = encode_maps16(cases[c], 0, cases[c]->pcur, &maps[8 * c], BATCH_PF_BOX_X, BATCH_PF_BOX_Y) &&
-                         encode_maps16(cases[c], 1, cases[c]->pcur, &maps[8 * c + 4], BATCH_PF_BOX_X, BATCH_PF_BOX_Y);
+                    ok = encode_maps16(cases[c], 0, 0, &maps[8 * c], BATCH_PF_BOX_X, BATCH_PF_BOX_Y) &&
+                         encode_maps16(cases[c], 1, 1, &maps[8 * c + 4], BATCH_PF_BOX_X, BATCH_PF_BOX_Y);
+#if LBM_DEBUG_CHECKS
+                std::vector<const void*> bases;
+                for (int c = 0; c < ncases; ++c)
+                    for (int k = 0; k < 2; ++k)
+                        for (const void* p : {(const void*)((char*)cases[c]->f[k] + 4 * cases[c]->N), (const void*)cases[c]->f[k],
+                                              (const void*)cases[c]->g[k], (const void*)cases[c]->phiu[k]})
+                            bases.push_back(p);
+                ok = ok && cudaMalloc(&b->d_bases, bases.size() * sizeof(void*)) == cudaSuccess &&
+                     cudaMemcpy(b->d_bases, bases.data(), bases.size() * sizeof(void*), cudaMemcpyHostToDevice) == cudaSuccess;
+                for (int cls = 0; cls < BATCH_NCLASS; ++cls)
+                    for (int k = 0; k < BATCH_NCAND; ++k) b->tab(cls, k).bases = b->d_bases;
+#endif
                 if (ok && cudaMalloc(&b->d_maps, maps.size() * sizeof(CUtensorMap)) == cudaSuccess &&
                     cudaMemcpy(b->d_maps, maps.data(), maps.size() * sizeof(CUtensorMap),
                                cudaMemcpyHostToDevice) == cudaSuccess) {

@@ -206,3 +206,28 @@ def test_batch_graphs_are_kept(libs, storage, n):
     finally:
         for lat in A + B:
             lat.close()
+
+
+def test_batch_prefetch_follows_the_phiu_buffer(libs):
+    """The index-checking build also checks that each prefetch map of a one-step
+    16-bit batch covers the buffer about to be read.  A several-step launch of one
+    case alone moves its (phi u) to the other buffer."""
+    lbm, release, debug = libs
+    _use(lbm, debug)
+    specs = cases.batch_cases(24, seed=11)
+    P = cases.params_static_drop()
+    specs.append(dict(nx=64, ny=64, params=P, phi0=cases.drop(64, 64, 16.0, P["W"]), ux0=None, uy0=None))
+    A = [lbm.Lattice(sp["nx"], sp["ny"], storage=1, check_every=1 << 20, **sp["params"])
+         .init(sp["phi0"], sp["ux0"], sp["uy0"]) for sp in specs]
+    try:
+        with lbm.Batch(A) as bt:
+            bt.step(3)
+            assert bt.counts()[0] == 6
+            A[24].step(3)
+            assert A[24].step_launches() == 1
+            bt.step(4)
+            A[24].init(specs[24]["phi0"])
+            bt.step(33)
+    finally:
+        for lat in A:
+            lat.close()
