@@ -38,8 +38,6 @@ UNIT = "MLUPS"
 # write 9 f + 9 g (72 B), read and write (phi u) of the previous step (16 B)
 BYTES_PER_LU = 160
 BYTES_PER_LU_POPULATIONS = 144
-# lbm_step takes two steps per read and write of the state on larger grids
-STEPS_PER_PASS = 2
 
 
 def _peaks():
@@ -275,6 +273,13 @@ def _time_steps(torch, stream, fn):
     return ev0.elapsed_time(ev1) / 1e3
 
 
+def passes_per_step(launches, steps, classes=1):
+    """Reads and writes of the whole state per step: each step launch is one, over
+    the cases of its boundary class (lbm_step and lbm_batch_step may take several
+    steps per launch)."""
+    return launches / (classes * steps)
+
+
 def run_batched(torch, lbm, stream, steps, storage=1):
     """The batched sweep: 64 independent drops and impacts of uneven sizes and
     parameters, each advanced `steps` steps (a) one case after another on the
@@ -305,8 +310,10 @@ def run_batched(torch, lbm, stream, steps, storage=1):
         lat.close()
     bat = make(storage)
     b = lbm.Batch(bat)
-    b.step(150)                                   # tile-shape tuning (140 steps) + warm-up
+    b.step(150)                                   # timing or tuning of its kernels + warm-up
+    n0 = b.counts()[0]
     t_bat = _time_steps(torch, stream, lambda: b.step(steps))
+    launches = b.counts()[0] - n0
     info = b.info()
     d_bat, u_bat = accuracy(bat)
     b.close()
@@ -324,8 +331,8 @@ def run_batched(torch, lbm, stream, steps, storage=1):
     v_bat = nodes * steps / t_bat / 1e6
     v_seq = nodes * steps / t_seq / 1e6
     peak, _ = _peaks()
-    # the batch takes two steps per pass over the state
-    bpl = (BYTES_PER_LU if storage == 0 else BYTES_PER_LU_SHIFTED16) / STEPS_PER_PASS
+    pps = passes_per_step(launches, steps, sum(info[k]["cases"] > 0 for k in ("periodic", "walls")))
+    bpl = (BYTES_PER_LU if storage == 0 else BYTES_PER_LU_SHIFTED16) * pps
     return {
         "cases": len(specs), "nodes": nodes, "steps_per_case": steps + 5,
         "storage": STORAGE_NAMES[storage], "value": v_bat, "unit": UNIT,
@@ -335,11 +342,11 @@ def run_batched(torch, lbm, stream, steps, storage=1):
         "tuned_us_per_step": {k: info[k]["us"] for k in ("periodic", "walls")},
         "bytes_per_lu": bpl,
         "roofline_frac": v_bat * 1e6 * bpl / 1e9 / peak,
-        "roofline_frac_88": (v_bat * 1e6 * BYTES_PER_LU_16_MIN / STEPS_PER_PASS / 1e9 / peak) if storage else None,
+        "roofline_frac_88": (v_bat * 1e6 * BYTES_PER_LU_16_MIN * pps / 1e9 / peak) if storage else None,
         "sum_phi_rel_drift_max": {"batched": max(d_bat), "sequential_fp32": max(d_seq)},
         "drop_umax_max": {"batched": max(u_bat[k] for k in drops),
                           "sequential_fp32": max(u_seq[k] for k in drops)},
-        "launches_per_step": 2 / STEPS_PER_PASS,  # one per boundary class and pass
+        "launches_per_step": launches / steps,
     }
 
 
@@ -352,14 +359,16 @@ def run_storage_variants(torch, lbm, stream, steps):
     for st in (1, 2, 3):
         lat = lbm.Lattice(nx, ny, stream=stream, storage=st, **params).init(phi0)
         lat.step(50)
+        n0 = lat.step_launches()
         t = _time_steps(torch, stream, lambda: lat.step(steps))
+        pps = passes_per_step(lat.step_launches() - n0, steps)
         lat.close()
         v = nx * ny * steps / t / 1e6
         peak, _ = _peaks()
         out[STORAGE_NAMES[st]] = {"value": v, "unit": UNIT,
-                                  "bytes_per_lu": BYTES_PER_LU_SHIFTED16 / STEPS_PER_PASS, "steps": steps,
-                                  "roofline_frac": v * 1e6 * BYTES_PER_LU_SHIFTED16 / STEPS_PER_PASS / 1e9 / peak,
-                                  "roofline_frac_88": v * 1e6 * BYTES_PER_LU_16_MIN / STEPS_PER_PASS / 1e9 / peak}
+                                  "bytes_per_lu": BYTES_PER_LU_SHIFTED16 * pps, "steps": steps,
+                                  "roofline_frac": v * 1e6 * BYTES_PER_LU_SHIFTED16 * pps / 1e9 / peak,
+                                  "roofline_frac_88": v * 1e6 * BYTES_PER_LU_16_MIN * pps / 1e9 / peak}
     return out
 
 
@@ -439,10 +448,11 @@ def run_ours(args):
 
     # -- device-resident throughput ------------------------------------------
     # one step per launch (LBM_KERNEL_GENERIC), the basis of 160 bytes per node and
-    # step; the default path, two steps per launch, is timed below
+    # step; the default path, several steps per launch, is timed below
     lat = lbm.Lattice(nx, ny, stream=stream, kernel=lbm.LBM_KERNEL_GENERIC, **params)
     lat.init(phi0)
     lat.step(args.warmup)
+    n_launch = lat.step_launches()
     torch.cuda.synchronize()
     barrier()
     torch.cuda.synchronize()
@@ -455,14 +465,18 @@ def run_ours(args):
     barrier()
     torch.cuda.synchronize()
     ms = ev0.elapsed_time(ev1)
+    n_launch = lat.step_launches() - n_launch
     s_phi, umax, _, _ = lat.diag()
     lat.close()
 
     # -- the default path: pairs of steps per launch ---------------------------
     lat = lbm.Lattice(nx, ny, stream=stream, **params).init(phi0)
     lat.step(args.warmup)
+    n_pairs = lat.step_launches()
     barrier()
     t_pairs = _time_steps(torch, stream, lambda: lat.step(args.steps))
+    n_pairs = lat.step_launches() - n_pairs
+    bpl_pairs = BYTES_PER_LU * passes_per_step(n_pairs, args.steps)
     lat.close()
 
     # -- end to end through the C ABI with host buffers ------------------------
@@ -529,13 +543,13 @@ def run_ours(args):
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": 8 * N / args.steps,
                     "d2h_bytes_per_step": 40 * N / args.steps},
             "clocks": clk.summary(),
-            "gpu_launches": args.steps,
+            "gpu_launches": n_launch,
             "two_steps_per_launch": {
                 "value": whole_job_mlups(N, args.steps, world, t_pairs), "unit": UNIT,
                 "ms_per_step": t_pairs * 1e3 / args.steps,
-                "gpu_launches": args.steps // STEPS_PER_PASS + args.steps % STEPS_PER_PASS,
-                "bytes_per_lu": BYTES_PER_LU / STEPS_PER_PASS,
-                "roofline_frac": BYTES_PER_LU / STEPS_PER_PASS * N * args.steps / t_pairs / 1e9 / peak,
+                "gpu_launches": n_pairs,
+                "bytes_per_lu": bpl_pairs,
+                "roofline_frac": bpl_pairs * N * args.steps / t_pairs / 1e9 / peak,
                 "kernel": "k_march (two steps per launch, FP32), the default of lbm_step"},
             "sum_phi": s_phi, "umax": umax,
             "batched": batched,

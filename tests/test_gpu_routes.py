@@ -231,3 +231,24 @@ def test_batch_prefetch_follows_the_phiu_buffer(libs):
     finally:
         for lat in A:
             lat.close()
+
+
+def test_bench_bytes_per_update_follow_the_launches(libs):
+    """bench.py's bytes per update of a batch are those of the launches it made:
+    half of a step's where the batch takes pairs (FP32 here), a whole step's
+    where it takes one-step launches."""
+    import torch
+
+    import bench
+
+    lbm, release, _ = libs
+    _use(lbm, release)
+    full = cases.batch_cases
+    cases.batch_cases = lambda n=64, seed=11: full(8, seed=11)
+    try:
+        s = torch.cuda.current_stream()
+        for storage, launches, bytes_ in ((0, 1.0, 80.0), (1, 2.0, 92.0)):
+            d = bench.run_batched(torch, lbm, s, 40, storage=storage)
+            assert d["cases"] == 8 and d["launches_per_step"] == launches and d["bytes_per_lu"] == bytes_
+    finally:
+        cases.batch_cases = full
