@@ -93,8 +93,10 @@ enum {
 /* step kernel (kernel) */
 enum {
     LBM_KERNEL_AUTO = 0,    /* the library's choice (by grid size and storage): lbm_step takes
-                               pairs of steps in one launch on larger grids; the same bits as
-                               LBM_KERNEL_GENERIC */
+                               two to six steps in one launch on small grids (up to about
+                               280^2), one on medium ones and pairs on large ones, as
+                               lbm_step_launches shows; the same bits as LBM_KERNEL_GENERIC.
+                               A captured stream takes one (see lbm_step) */
     LBM_KERNEL_GENERIC = 1  /* one step per launch: tiles of 32 x 4 threads, direct loads, phi ring recomputed
                                in shared memory; one node per thread with FP32 storage,
                                two with 16-bit storage; any grid */

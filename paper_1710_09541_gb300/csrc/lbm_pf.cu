@@ -1031,9 +1031,13 @@ static MarchKernel march_kernel(const lbm_params& p, size_t* smem) {
 // enough.  One-step time / march time at eff, nx a multiple of 8: FP32 640^2 0.47
 // 0.94, 768^2 0.54 1.09, 896^2 0.61 1.29, 1024^2 0.67 1.32; FP16 896^2 0.61 0.95, 1024^2
 // 0.67 0.98, 1152^2 0.71 1.05, 1280^2 0.75 1.10, walled 800 x 500 0.48 0.92, 1200 x 700
-// 0.65 1.04, 2400 x 600 0.75 1.08.  Other nx, whose rows start inside a 32-byte sector,
-// slow the one-step kernels down: FP32 501^2 0.36 1.14, 901 x 300 0.41 1.17; FP16 901 x
-// 300 0.41 0.97, 601^2 0.47 1.14, 801^2 0.58 1.10, 1001^2 0.66 1.01, 1501 x 1103 0.74 1.15.
+// 0.65 1.04, 2400 x 600 0.75 1.08; walled FP32 640^2 0.47 0.99, 800 x 500 0.48 1.04, 704^2
+// 0.54 1.01, 768^2 0.54 1.16.  Other nx, whose rows start inside a 32-byte sector,
+// slow the one-step kernels down: FP32 501^2 0.36 1.15, 901 x 300 0.41 1.17 (walled 1.15,
+// 1.18); FP16 901 x 300 0.41 0.97, 601^2 0.47 1.14, 801^2 0.58 1.10, 1001^2 0.66 1.01, 1501 x
+// 1103 0.74 1.15.  The FP32 line of these, 0.36, is the lowest point it was first tried
+// at and no crossover: periodic grids gain below it too (351^2 0.27 1.20, 401^2 0.29
+// 1.07, 451^2 0.32 1.24, 801 x 151 0.27 1.17), a walled 401^2 nothing (1.00).
 static MarchGrid plan_march(int nx, int ny, const lbm_params& p, int sms) {
     MarchGrid g = {0, 0, 0};
     if (p.kernel == LBM_KERNEL_GENERIC || nx < 64 || ny < 16) return g;
